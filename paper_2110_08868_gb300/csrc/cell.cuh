@@ -89,6 +89,7 @@ struct Poly {
         };
     };
     float sup[27];            // support max_v v.u over the 26 stencil directions u
+    float supi[27];           // the same inflated for the certificate (cert_sup)
     int np, nt;
     int ncert;                // seeds recorded for the cell's certificate (-1: too many)
 #ifdef SDOT_COUNTERS
@@ -803,7 +804,7 @@ __device__ __forceinline__ float circ_gap(float p, float lo, float w, float Lt) 
     return fminf(t - w, Lt - t);
 }
 
-// True when no seed of node (X, Y, Z) of a pyramid level can cut the polytope:
+// A node (X, Y, Z) of a pyramid level is pruned when no seed in it can cut the polytope:
 // 1/2 (u - Rc)_+^2 >= Mv + psimax - psi_i with u the distance from the ball centre
 // to the node's box (see the head of this file). The level (its psimax row pmax, node
 // counts d and node size sz) and the ball (centre c in absolute coordinates, Rc, Mv,
@@ -824,11 +825,12 @@ __device__ __forceinline__ WalkBall walk_ball(const Bounds& b) {
     return w;
 }
 
-__device__ __forceinline__ bool node_pruned(const float* __restrict__ pmax, const int d[3],
+// Returns the node's psimax when it must be opened, -inf when it is pruned.
+__device__ __forceinline__ float node_bound(const float* __restrict__ pmax, const int d[3],
                                             const float sz[3], const float Lt[3],
                                             const WalkBall& wb, int X, int Y, int Z) {
     const float pm = pmax[(int64_t)((Z * d[1] + Y) * d[0] + X)];
-    if (pm == -INFINITY) return true;  // no seed inside
+    if (pm == -INFINITY) return pm;  // no seed inside
     const int c[3] = {X, Y, Z};
     float u2 = 0.f;
 #pragma unroll
@@ -843,7 +845,7 @@ __device__ __forceinline__ bool node_pruned(const float* __restrict__ pmax, cons
     const float lhs = 0.5f * du * du;
     const float rhs = wb.Mv + (pm - wb.psi_i);
     const float margin = 2e-5f * (lhs + wb.Mv + fabsf(pm) + fabsf(wb.psi_i)) + 1e-5f;
-    return lhs - rhs > margin;
+    return lhs - rhs > margin ? -INFINITY : pm;
 }
 
 // Conservative FP32 test: can the plane (n, w) of a seed (seed frame) reach the
@@ -854,16 +856,24 @@ __device__ __forceinline__ bool node_pruned(const float* __restrict__ pmax, cons
 // so by sublinearity of the support h, h(n) <= n3 h(u3) + (n2 - n3) h(u2) +
 // (n1 - n2) h(u1); this is never weaker than the bounding box's support. (2) The ball
 // of radius Rc around the box centre c: h(n) <= c.n + Rc |n|.
-__device__ __forceinline__ bool support_may_cut(const float* sup, const Bounds& b, float nx,
-                                                float ny, float nz, float w) {
-    float m[3] = {fabsf(nx), fabsf(ny), fabsf(nz)};
+struct SortedNormal {
+    float m[3];   // |n| sorted, descending
+    int k[3];     // stencil directions u1, u2, u3
+    float cn, ln; // c.n and |n|
+};
+
+__device__ __forceinline__ SortedNormal sort_normal(const Bounds& b, float nx, float ny, float nz) {
+    SortedNormal q;
+    q.m[0] = fabsf(nx);
+    q.m[1] = fabsf(ny);
+    q.m[2] = fabsf(nz);
     int code[3] = {nx >= 0.f ? 1 : -1, ny >= 0.f ? 3 : -3, nz >= 0.f ? 9 : -9};
     // sort descending (three compare-exchanges)
 #define SDOT_CX(i, j)                                  \
-    if (m[i] < m[j]) {                                 \
-        const float tm = m[i];                         \
-        m[i] = m[j];                                   \
-        m[j] = tm;                                     \
+    if (q.m[i] < q.m[j]) {                             \
+        const float tm = q.m[i];                       \
+        q.m[i] = q.m[j];                               \
+        q.m[j] = tm;                                   \
         const int tc = code[i];                        \
         code[i] = code[j];                             \
         code[j] = tc;                                  \
@@ -872,15 +882,22 @@ __device__ __forceinline__ bool support_may_cut(const float* sup, const Bounds& 
     SDOT_CX(1, 2)
     SDOT_CX(0, 1)
 #undef SDOT_CX
-    const int k1 = 13 + code[0], k2 = k1 + code[1], k3 = k2 + code[2];
-    const float t3 = m[2] * sup[k3], t2 = (m[1] - m[2]) * sup[k2], t1 = (m[0] - m[1]) * sup[k1];
+    q.k[0] = 13 + code[0];
+    q.k[1] = q.k[0] + code[1];
+    q.k[2] = q.k[1] + code[2];
+    q.cn = b.c[0] * nx + b.c[1] * ny + b.c[2] * nz;
+    q.ln = sqrtf(nx * nx + ny * ny + nz * nz);
+    return q;
+}
+
+__device__ __forceinline__ bool reaches(const SortedNormal& q, const float* sup, float Rc, float w) {
+    const float t3 = q.m[2] * sup[q.k[2]], t2 = (q.m[1] - q.m[2]) * sup[q.k[1]],
+                t1 = (q.m[0] - q.m[1]) * sup[q.k[0]];
     const float S = t1 + t2 + t3;
     const float margin = 2e-5f * (fabsf(t1) + fabsf(t2) + fabsf(t3) + fabsf(w)) + 1e-5f;
-    if (!(S > w - margin)) return false;
-    const float cn = b.c[0] * nx + b.c[1] * ny + b.c[2] * nz;
-    const float rn = b.Rc * sqrtf(nx * nx + ny * ny + nz * nz);
-    const float margin2 = 2e-5f * (fabsf(cn) + rn + fabsf(w)) + 1e-5f;
-    return cn + rn > w - margin2;
+    const float rn = Rc * q.ln;
+    const float margin2 = 2e-5f * (fabsf(q.cn) + rn + fabsf(w)) + 1e-5f;
+    return S > w - margin && q.cn + rn > w - margin2;
 }
 
 // Carried security certificates. A pass-1 walk that certifies a cell records, besides
@@ -900,38 +917,6 @@ constexpr float CERT_ETA = 0.01f;  // reserve for the change of psi_j - psi_i, u
 // inflated support of direction k as stored (FP16, rounded up)
 __device__ __forceinline__ float cert_sup(const float* sup, int k) {
     return __half2float(__float2half_ru(__fadd_ru(sup[k], CERT_EPS)));
-}
-
-// The prefilter of support_may_cut on the inflated certificate quantities.
-__device__ __forceinline__ bool cert_may_cut(const float* sup, const Bounds& b, float nx,
-                                             float ny, float nz, float w) {
-    float m[3] = {fabsf(nx), fabsf(ny), fabsf(nz)};
-    int code[3] = {nx >= 0.f ? 1 : -1, ny >= 0.f ? 3 : -3, nz >= 0.f ? 9 : -9};
-#define SDOT_CX(i, j)                                  \
-    if (m[i] < m[j]) {                                 \
-        const float tm = m[i];                         \
-        m[i] = m[j];                                   \
-        m[j] = tm;                                     \
-        const int tc = code[i];                        \
-        code[i] = code[j];                             \
-        code[j] = tc;                                  \
-    }
-    SDOT_CX(0, 1)
-    SDOT_CX(1, 2)
-    SDOT_CX(0, 1)
-#undef SDOT_CX
-    const int k1 = 13 + code[0], k2 = k1 + code[1], k3 = k2 + code[2];
-    const float t3 = m[2] * cert_sup(sup, k3), t2 = (m[1] - m[2]) * cert_sup(sup, k2),
-                t1 = (m[0] - m[1]) * cert_sup(sup, k1);
-    const float wr = __fsub_rd(w, CERT_ETA);
-    const float S = t1 + t2 + t3;
-    const float margin = 2e-5f * (fabsf(t1) + fabsf(t2) + fabsf(t3) + fabsf(wr)) + 1e-5f;
-    if (!(S > wr - margin)) return false;
-    const float R = __fadd_ru(b.Rc, CERT_EPS);
-    const float cn = b.c[0] * nx + b.c[1] * ny + b.c[2] * nz;
-    const float rn = R * sqrtf(nx * nx + ny * ny + nz * nz);
-    const float margin2 = 2e-5f * (fabsf(cn) + rn + fabsf(wr)) + 1e-5f;
-    return cn + rn > wr - margin2;
 }
 
 enum { MODE_CERTIFY = 0, MODE_FULL = 1 };
@@ -977,14 +962,164 @@ __device__ __forceinline__ V4<R> shfl_plane(const V4<R>& p, int src) {
     return q;
 }
 
-// The seeds of up to 32 grid cells (leaf < 0: none), spread evenly over the lanes:
-// each seed passes the conservative prefilter in its lane, the survivors are checked
-// exactly one by one (warp-uniform). CERTIFY stops at the first seed that cuts; FULL
-// clips it. Returns LEAF_STOP when the cell's processing must stop.
+// Is seed j one of the polytope's planes, from the lane's copies of P.pj (lane j holds
+// slots j, j + 32, ...; -1 beyond the last)? (warp-uniform j)
+template <typename R, class C>
+__device__ __forceinline__ void load_planes(const Poly<R, C>& P, int32_t (&pj)[C::NW], int lane) {
+#pragma unroll
+    for (int q = 0; q < C::NW; q++) pj[q] = lane + 32 * q < P.np ? P.pj[lane + 32 * q] : -1;
+}
+template <int NW>
+__device__ __forceinline__ bool among(const int32_t (&pj)[NW], int32_t j) {
+    bool d = false;
+#pragma unroll
+    for (int q = 0; q < NW; q++) d |= pj[q] == j;
+    return __any_sync(FULLMASK, d);
+}
+
+// Per lane: can the FP32 plane (seed frame) reach a vertex? Conservative like the
+// prefilter: it may differ from the exact plane by the margin.
+template <typename R, class C>
+__device__ __noinline__ bool reaches_vertex(const Poly<R, C>& P, const Bounds& b, float nx, float ny,
+                                            float nz, float w) {
+    const float z0 = b.zf[0], z1 = b.zf[1], z2 = b.zf[2];
+    float h = -INFINITY;
+#pragma unroll 1
+    for (int s = 0; s < P.nt; s++) {
+        const float x = (float)P.vx[s] + z0, y = (float)P.vy[s] + z1, z = (float)P.vz[s] + z2;
+        h = fmaxf(h, fmaf(nx, x, fmaf(ny, y, nz * z)));
+    }
+    const float margin =
+        2e-5f * ((fabsf(nx) + fabsf(ny) + fabsf(nz)) * sqrtf(2.f * b.Mv) + fabsf(w)) + 1e-5f;
+    return h > w - margin;
+}
+
+// Candidates left in a round from which the per-lane vertex test pays: it costs about as
+// much as six exact tests, which the warp runs one after the other.
+constexpr int VERTEX_TEST_MIN = 7;
+
+// The seeds of every lane's two runs [s0, s0 + n0) and [s1, s1 + n1) of the sorted order,
+// spread evenly over the lanes: each seed passes the conservative prefilter in its lane,
+// the survivors are checked exactly one by one (warp-uniform). CERTIFY stops at the first
+// seed that cuts; FULL clips it. Returns LEAF_STOP when the cell's processing must stop.
 template <typename R, class C, int MODE>
-__device__ __noinline__ int process_leaves(Poly<R, C>& P, const ClipParams& cp,
-                                           const CellCtx& cc, Bounds& b, int64_t leaf, int lane,
-                                           bool& bad, uint32_t& st) {
+__device__ __noinline__ int process_seeds(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
+                                          Bounds& b, int32_t s0, int n0, int32_t s1, int n1,
+                                          int lane, bool& bad, uint32_t& st) {
+    const int n = n0 + n1;
+    int incl = n;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULLMASK, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(FULLMASK, incl, 31);
+    const int excl = incl - n;
+    const int32_t first = s0 - excl, jump = s1 - (s0 + n0);
+    const int split = excl + n0;
+    WCOUNT(P, 4, total);
+    // a certifying walk of the first pass records the cell's certificate
+    const bool rec = MODE == MODE_CERTIFY && cp.pass == 1 && cp.cert_use;
+    int32_t pj[C::NW];
+    load_planes(P, pj, lane);
+    for (int base = 0; base < total; base += 32) {
+        const int t = base + lane;
+        // the lane q owning flattened seed t: the first with incl[q] > t
+        int q = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const int y = __shfl_sync(FULLMASK, incl, q + step - 1);
+            if (y <= t) q += step;
+        }
+        int32_t s = t + __shfl_sync(FULLMASK, first, q);
+        const int sp = __shfl_sync(FULLMASK, split, q);
+        const int32_t jq = __shfl_sync(FULLMASK, jump, q);
+        if (t >= sp) s += jq;
+        bool cand = false, nearb = false;
+        float nx = 0.f, ny = 0.f, nz = 0.f, w = 0.f;
+        if (t < total && s != (int32_t)cc.i) {
+            plane_f32(cp, cc.si, s, nx, ny, nz, w);
+            const SortedNormal sn = sort_normal(b, nx, ny, nz);
+            cand = reaches(sn, P.sup, b.Rc, w);
+            if (rec)
+                nearb = cand || reaches(sn, P.supi, __fadd_ru(b.Rc, CERT_EPS), __fsub_rd(w, CERT_ETA));
+        }
+        uint32_t cm = __ballot_sync(FULLMASK, cand);
+        uint32_t nm = rec ? __ballot_sync(FULLMASK, nearb) : cm;
+        WCOUNT(P, 5, __popc(cm));
+        if (!nm) continue;
+        // drop the seeds that already are planes of the polytope (the cell's own facet
+        // neighbours pass the prefilter), then build the exact planes of the rest
+        for (uint32_t m2 = nm; m2;) {
+            const int src = __ffs(m2) - 1;
+            m2 &= m2 - 1;
+            if (among(pj, __shfl_sync(FULLMASK, s, src))) {
+                cm &= ~(1u << src);
+                nm &= ~(1u << src);
+            }
+        }
+        // the certificate's seeds to re-test (P.ftri is free during a certifying walk)
+        if (rec && nm) {
+            const int c0 = P.ncert;
+            const int k = __popc(nm);
+            __syncwarp();
+            if (c0 >= 0 && c0 + k <= CERT_NEAR) {
+                if ((nm >> lane) & 1u) P.ftri[c0 + __popc(nm & lanes_below(lane))] = (uint32_t)s;
+                if (lane == 0) P.ncert = c0 + k;
+            } else if (lane == 0) {
+                P.ncert = -1;
+            }
+            __syncwarp();
+        }
+        if (__popc(cm) >= VERTEX_TEST_MIN) {
+            cand = ((cm >> lane) & 1u) && reaches_vertex(P, b, nx, ny, nz, w);
+            cm = __ballot_sync(FULLMASK, cand);
+        }
+        if (!cm) continue;
+        cand = (cm >> lane) & 1u;
+        V4<R> pl;
+        pl.x = pl.y = pl.z = pl.w = R(0);
+        R len = R(1);
+        if (cand) build_plane(cp, cc, s, pl, len);
+        bool cut = false;
+        while (cm) {
+            const int src = __ffs(cm) - 1;
+            cm &= cm - 1;
+            const V4<R> pn = shfl_plane(pl, src);
+            const R plen = __shfl_sync(FULLMASK, len, src);
+            if (MODE == MODE_CERTIFY) {
+                if (poly_cut_by(P, pn, plen, lane)) {
+                    st |= CS_UNCERTIFIED;
+                    return LEAF_STOP;
+                }
+                continue;
+            }
+            const int32_t j = __shfl_sync(FULLMASK, s, src);
+            const int rc = poly_clip(P, pn, plen, j, lane, bad);
+            if (rc == CLIP_EMPTY) {
+                st |= CS_EMPTY;
+                return LEAF_STOP;
+            }
+            if (rc == CLIP_CAP) {
+                st |= CS_CAPACITY | CS_CAP_POLY;
+                return LEAF_STOP;
+            }
+            cut |= rc == CLIP_CUT;
+        }
+        // the bounds of this round's start stay valid (larger) for its later seeds, whose
+        // exact test decides; the next round starts from the smaller polytope
+        if (MODE == MODE_FULL && cut) {
+            poly_bounds(P, cp, b, lane);
+            load_planes(P, pj, lane);
+        }
+    }
+    return LEAF_OK;
+}
+
+// the seeds of up to 32 grid cells (leaf < 0: none)
+template <typename R, class C, int MODE>
+__device__ __forceinline__ int process_leaves(Poly<R, C>& P, const ClipParams& cp,
+                                              const CellCtx& cc, Bounds& b, int64_t leaf, int lane,
+                                              bool& bad, uint32_t& st) {
     int32_t sb = 0;
     int n = 0;
     if (leaf >= 0) {
@@ -997,102 +1132,11 @@ __device__ __noinline__ int process_leaves(Poly<R, C>& P, const ClipParams& cp,
         WCOUNT(P, 3, nleaf);
     }
 #endif
-    int incl = n;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULLMASK, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(FULLMASK, incl, 31);
-    const int excl = incl - n;
-    WCOUNT(P, 4, total);
-    // a certifying walk of the first pass records the cell's certificate
-    const bool rec = MODE == MODE_CERTIFY && cp.pass == 1 && cp.cert_use;
-    for (int base = 0; base < total; base += 32) {
-        const int t = base + lane;
-        // the lane q owning flattened seed t: the first with incl[q] > t
-        int q = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-            const int y = __shfl_sync(FULLMASK, incl, q + step - 1);
-            if (y <= t) q += step;
-        }
-        const int ex = __shfl_sync(FULLMASK, excl, q);
-        const int32_t s0 = __shfl_sync(FULLMASK, sb, q);
-        const int32_t s = s0 + (t - ex);
-        bool cand = false, nearb = false;
-        if (t < total && s != (int32_t)cc.i) {
-            float nx, ny, nz, w;
-            plane_f32(cp, cc.si, s, nx, ny, nz, w);
-            cand = support_may_cut(P.sup, b, nx, ny, nz, w);
-            if (rec) nearb = cand || cert_may_cut(P.sup, b, nx, ny, nz, w);
-        }
-        uint32_t cm = __ballot_sync(FULLMASK, cand);
-        uint32_t nm = rec ? __ballot_sync(FULLMASK, nearb) : cm;
-        WCOUNT(P, 5, __popc(cm));
-        if (!nm) continue;
-        // drop the seeds that already are planes of the polytope (the cell's own facet
-        // neighbours pass the prefilter), then build the exact planes of the rest
-        for (uint32_t m2 = nm; m2;) {
-            const int src = __ffs(m2) - 1;
-            m2 &= m2 - 1;
-            if (has_plane(P, __shfl_sync(FULLMASK, s, src), lane)) {
-                cm &= ~(1u << src);
-                nm &= ~(1u << src);
-            }
-        }
-        // the certificate's seeds to re-test (P.ftri is free during a certifying walk)
-        if (rec && nm) {
-            const int n0 = P.ncert;
-            const int k = __popc(nm);
-            __syncwarp();
-            if (n0 >= 0 && n0 + k <= CERT_NEAR) {
-                if ((nm >> lane) & 1u) P.ftri[n0 + __popc(nm & lanes_below(lane))] = (uint32_t)s;
-                if (lane == 0) P.ncert = n0 + k;
-            } else if (lane == 0) {
-                P.ncert = -1;
-            }
-            __syncwarp();
-        }
-        if (!cm) continue;
-        cand = (cm >> lane) & 1u;
-        V4<R> pl;
-        pl.x = pl.y = pl.z = pl.w = R(0);
-        R len = R(1);
-        if (cand) build_plane(cp, cc, s, pl, len);
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1;
-            const int32_t j = __shfl_sync(FULLMASK, s, src);
-            const V4<R> pn = shfl_plane(pl, src);
-            const R plen = __shfl_sync(FULLMASK, len, src);
-            // an earlier clip of this round may have added the same seed? (seeds are
-            // distinct within a round, so only FULL mode's clips can change the set)
-            if (MODE == MODE_FULL && has_plane(P, j, lane)) continue;
-            if (MODE == MODE_CERTIFY) {
-                if (poly_cut_by(P, pn, plen, lane)) {
-                    st |= CS_UNCERTIFIED;
-                    return LEAF_STOP;
-                }
-                continue;
-            }
-            const int rc = poly_clip(P, pn, plen, j, lane, bad);
-            if (rc == CLIP_EMPTY) {
-                st |= CS_EMPTY;
-                return LEAF_STOP;
-            }
-            if (rc == CLIP_CAP) {
-                st |= CS_CAPACITY | CS_CAP_POLY;
-                return LEAF_STOP;
-            }
-            if (rc == CLIP_CUT) poly_bounds(P, cp, b, lane);
-        }
-    }
-    return LEAF_OK;
+    return process_seeds<R, C, MODE>(P, cp, cc, b, sb, n, sb + n, 0, lane, bad, st);
 }
 
 // Near-first pass for re-queued cells: the grid cells in Chebyshev rings around the
-// grid cell of the previous centroid, so the polytope is small before the pyramid
-// walk (which visits nodes in no particular order) starts.
+// grid cell of the previous centroid, so the polytope is small before the walk starts.
 template <typename R, class C>
 __device__ __noinline__ bool ring_walk(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
                                        Bounds& b, const float* zprev, int lane, bool& bad,
@@ -1111,17 +1155,24 @@ __device__ __noinline__ bool ring_walk(Poly<R, C>& P, const ClipParams& cp, cons
         if (2 * r + 1 > Gmin) break;
         if (r >= 2 && (float)(r - 1) * hmin > 2.f * b.Rc) break;
         const int w = 2 * r + 1, n3 = w * w * w;
+        const float iw = 1.f / (float)w, iw2 = iw * iw;
+#pragma unroll 1
         for (int base = 0; base < n3; base += 32) {
             const int t = base + lane;
             int64_t leaf = -1;
             if (t < n3) {
-                const int ox = t % w - r, oy = (t / w) % w - r, oz = t / (w * w) - r;
-                const int ch = max(abs(ox), max(abs(oy), abs(oz)));
+                // t = x + w (y + w z), quotients exact for these small numbers
+                const int z = (int)(((float)t + 0.5f) * iw2), tz = t - z * w * w;
+                const int y = (int)(((float)tz + 0.5f) * iw), x = tz - y * w;
+                const int ch = max(abs(x - r), max(abs(y - r), abs(z - r)));
                 if (ch == r) {
-                    const int cx = ((ca[0] + ox) % cp.G[0] + cp.G[0]) % cp.G[0];
-                    const int cy = ((ca[1] + oy) % cp.G[1] + cp.G[1]) % cp.G[1];
-                    const int cz = ((ca[2] + oz) % cp.G[2] + cp.G[2]) % cp.G[2];
-                    leaf = ((int64_t)cz * cp.G[1] + cy) * cp.G[0] + cx;
+                    int c[3] = {ca[0] + x - r, ca[1] + y - r, ca[2] + z - r};
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {  // at most one period away (w <= G)
+                        if (c[a] < 0) c[a] += cp.G[a];
+                        else if (c[a] >= cp.G[a]) c[a] -= cp.G[a];
+                    }
+                    leaf = ((int64_t)c[2] * cp.G[1] + c[1]) * cp.G[0] + c[0];
                 }
             }
             if (process_leaves<R, C, MODE_FULL>(P, cp, cc, b, leaf, lane, bad, st) == LEAF_STOP)
@@ -1140,18 +1191,24 @@ __device__ __forceinline__ uint32_t pack_node(int l, int x, int y, int z) {
     return ((uint32_t)l << 27) | ((uint32_t)z << 18) | ((uint32_t)y << 9) | (uint32_t)x;
 }
 
+// The ball of a walk; a recording walk takes it with the certificate's reserves (the same
+// roundings as cert_store).
+__device__ __forceinline__ WalkBall walk_ball(const Bounds& b, bool rec) {
+    WalkBall wb = walk_ball(b);
+    if (rec) {
+        wb.Rc = __fadd_ru(wb.Rc, CERT_EPS);
+        wb.Mv = __fadd_ru(wb.Mv, CERT_ETA);
+    }
+    return wb;
+}
+
 template <typename R, class C, int MODE>
 __device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
                                       Bounds& b, int lane, bool& bad, uint32_t& st) {
     if (lane == 0) P.stack[0] = pack_node(cp.pyr.nlev, 0, 0, 0);
     int sp = 1;
     const float Lt[3] = {cp.Lt[0], cp.Lt[1], cp.Lt[2]};
-    WalkBall wb = walk_ball(b);
-    if (MODE == MODE_CERTIFY && cp.pass == 1 && cp.cert_use) {
-        // the certificate's reserves (the same roundings as cert_store)
-        wb.Rc = __fadd_ru(wb.Rc, CERT_EPS);
-        wb.Mv = __fadd_ru(wb.Mv, CERT_ETA);
-    }
+    WalkBall wb = walk_ball(b, MODE == MODE_CERTIFY && cp.pass == 1 && cp.cert_use);
     __syncwarp();
     while (sp > 0) {
         const uint32_t e = P.stack[sp - 1];
@@ -1171,7 +1228,7 @@ __device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const
             const int cx = x0 + (t & 3), cy = y0 + ((t >> 2) & 3), cz = z0 + (t >> 4);
             bool surv = false;
             if (cx < cd[0] && cy < cd[1] && cz < cd[2])
-                surv = !node_pruned(pmax, cd, csz, Lt, wb, cx, cy, cz);
+                surv = node_bound(pmax, cd, csz, Lt, wb, cx, cy, cz) != -INFINITY;
             WCOUNT(P, 2, 32);
             const uint32_t sm = __ballot_sync(FULLMASK, surv);
             if (sm == 0) continue;
@@ -1190,10 +1247,128 @@ __device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const
             const int64_t leaf = surv ? ((int64_t)cz * cp.G[1] + cy) * cp.G[0] + cx : -1;
             if (process_leaves<R, C, MODE>(P, cp, cc, b, leaf, lane, bad, st) == LEAF_STOP)
                 return false;
-            if (MODE == MODE_FULL) wb = walk_ball(b);  // a clip may have shrunk the polytope
+            if (MODE == MODE_FULL) wb = walk_ball(b, false);  // a clip may have shrunk the polytope
         }
     }
     return true;
+}
+
+// The certifying walk by a window. The pyramid is walked down to level 1 only (nodes of
+// 4 x 4 x 4 grid cells); with psimax the largest bound among the level-1 nodes left, no
+// seed beyond U = Rc + sqrt(2 (Mv + psimax - psi_i)) from the ball's centre can cut. The
+// grid cells within U are taken row by row: the cells of a row are consecutive in the
+// sorted order, so a lane's row is one run of seeds (two where it wraps), and the rounds
+// over the seeds are full. Walking the pyramid to the grid cells opened about 12 nodes a
+// cell, whose rounds held 3 cells and 7 seeds each for 32 lanes: the walk of a certified
+// cell took 264 k cycles of its warp (97^3 to 129^3 boxes), by the window 124-163 k. With the
+// vertex test of process_seeds, an evaluation of a solved clumpy 33^3 box went from 8.6
+// to 4.4 ms for a trial and an accepted step, a clumpy 35^3 solve from 442 to 281 ms.
+// Returns WALK_DONE, WALK_STOP (a seed cuts), or WALK_OTHER when the window would hold
+// more than WINDOW_CELLS grid cells or wrap onto itself: the caller then walks the
+// pyramid. (A psimax far above its surroundings, next to a clump, widens the window for
+// every direction, where the pyramid opens only the nodes that need it.)
+enum { WALK_DONE = 0, WALK_STOP = 1, WALK_OTHER = 2 };
+constexpr int WINDOW_CELLS = 1000;
+
+template <typename R, class C>
+__device__ __noinline__ int window_walk(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
+                                        Bounds& b, int lane, bool& bad, uint32_t& st) {
+    if (cp.pyr.nlev < 2) return WALK_OTHER;
+    if (lane == 0) P.stack[0] = pack_node(cp.pyr.nlev, 0, 0, 0);
+    int sp = 1;
+    const float Lt[3] = {cp.Lt[0], cp.Lt[1], cp.Lt[2]};
+    const WalkBall wb = walk_ball(b, cp.pass == 1 && cp.cert_use);
+    float pm = -INFINITY;
+    __syncwarp();
+    while (sp > 0) {
+        const uint32_t e = P.stack[sp - 1];
+        sp--;
+        __syncwarp();
+        const int cl = (int)(e >> 27) - 1;  // level of the children
+        const int x0 = 4 * (int)(e & 511u), y0 = 4 * (int)((e >> 9) & 511u),
+                  z0 = 4 * (int)((e >> 18) & 511u);
+        const int cd[3] = {cp.pyr.dim[cl][0], cp.pyr.dim[cl][1], cp.pyr.dim[cl][2]};
+        const float csz[3] = {cp.nsz[cl][0], cp.nsz[cl][1], cp.nsz[cl][2]};
+        const float* pmax = cp.pyr.psimax + cp.pyr.off[cl];
+        const int nzr = min(4, cd[2] - z0);
+        WCOUNT(P, 7, 1);
+#pragma unroll 1
+        for (int base = 0; base < 16 * nzr; base += 32) {
+            const int t = base + lane;
+            const int cx = x0 + (t & 3), cy = y0 + ((t >> 2) & 3), cz = z0 + (t >> 4);
+            float nb = -INFINITY;
+            if (cx < cd[0] && cy < cd[1] && cz < cd[2])
+                nb = node_bound(pmax, cd, csz, Lt, wb, cx, cy, cz);
+            WCOUNT(P, 2, 32);
+            if (cl == 1) {
+                pm = fmaxf(pm, nb);
+                continue;
+            }
+            const uint32_t sm = __ballot_sync(FULLMASK, nb != -INFINITY);
+            const int n = __popc(sm);
+            if (sp + n > C::STK) return WALK_OTHER;
+            if (nb != -INFINITY) P.stack[sp + __popc(sm & lanes_below(lane))] = pack_node(cl, cx, cy, cz);
+            sp += n;
+            __syncwarp();
+        }
+    }
+    pm = warp_max(pm);
+    if (pm == -INFINITY) return WALK_DONE;
+    const float rhs = fmaxf(wb.Mv + (pm - wb.psi_i), 0.f);
+    const float slack = 2e-5f * (2.f * rhs + wb.Mv + fabsf(pm) + fabsf(wb.psi_i)) + 2e-5f;
+    // 1e-3: rounding of the grid cell edges in absolute FP32 coordinates
+    const float U = (wb.Rc + sqrtf(2.f * (rhs + slack))) * 1.0001f + 1e-3f;
+    float lo[3];
+    int w[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float ih = 1.f / cp.ht[a];
+        lo[a] = floorf((wb.c[a] - U) * ih);
+        const float width = floorf((wb.c[a] + U) * ih) - lo[a] + 1.f;
+        if (!(width <= (float)cp.G[a])) return WALK_OTHER;
+        w[a] = (int)width;
+    }
+    if (w[0] * w[1] * w[2] > WINDOW_CELLS) return WALK_OTHER;
+    const int rows = w[1] * w[2];
+    const float iw = 1.f / (float)w[1], ihx = 1.f / cp.ht[0];
+#pragma unroll 1
+    for (int base = 0; base < rows; base += 32) {
+        const int row = base + lane;
+        int32_t s0 = 0, s1 = 0;
+        int n0 = 0, n1 = 0;
+        if (row < rows) {
+            const int rz = (int)(((float)row + 0.5f) * iw), ry = row - rz * w[1];
+            const float Y = lo[1] + (float)ry, Z = lo[2] + (float)rz;
+            const float ay = fmaf(Y, cp.ht[1], -wb.c[1]), az = fmaf(Z, cp.ht[2], -wb.c[2]);
+            const float gy = fmaxf(fmaxf(ay, -ay - cp.ht[1]), 0.f),
+                        gz = fmaxf(fmaxf(az, -az - cp.ht[2]), 0.f);
+            const float rem = U * U - gy * gy - gz * gz;
+            if (rem >= 0.f) {
+                const float half = sqrtf(rem);
+                int X0 = (int)floorf((wb.c[0] - half) * ihx), X1 = (int)floorf((wb.c[0] + half) * ihx);
+                int cy = (int)Y, cz = (int)Z;
+                if (cy < 0) cy += cp.G[1];
+                else if (cy >= cp.G[1]) cy -= cp.G[1];
+                if (cz < 0) cz += cp.G[2];
+                else if (cz >= cp.G[2]) cz -= cp.G[2];
+                if (X0 < 0) {
+                    X0 += cp.G[0];
+                    X1 += cp.G[0];
+                }
+                const int32_t* cs = cp.cell_start + ((int64_t)cz * cp.G[1] + cy) * cp.G[0];
+                s0 = cs[X0];
+                n0 = cs[min(X1, cp.G[0] - 1) + 1] - s0;
+                if (X1 >= cp.G[0]) {
+                    s1 = cs[0];
+                    n1 = cs[X1 - cp.G[0] + 1] - s1;
+                }
+            }
+        }
+        if (process_seeds<R, C, MODE_CERTIFY>(P, cp, cc, b, s0, n0, s1, n1, lane, bad, st) ==
+            LEAF_STOP)
+            return WALK_STOP;
+    }
+    return WALK_DONE;
 }
 
 // Integrate the polytope and write the outputs of cell i; cen receives the centroid
@@ -1657,7 +1832,7 @@ __device__ __noinline__ void cert_store(const Poly<R, C>& P, const ClipParams& c
                                         int64_t i, int lane) {
     if (lane < 27)
         cp.cert_s[i * CERT_S + lane] =
-            lane == 13 ? (uint16_t)0 : __half_as_ushort(__float2half_ru(__fadd_ru(P.sup[lane], CERT_EPS)));
+            lane == 13 ? (uint16_t)0 : __half_as_ushort(__float2half_ru(P.supi[lane]));
     const int n = P.ncert;
     if (lane < n) cp.cert_j[i * CERT_NEAR + lane] = (int32_t)P.ftri[lane];
     if (lane == 0) {
@@ -1737,6 +1912,7 @@ __device__ __forceinline__ bool process_cell(Poly<R, C>& P, const ClipParams& cp
         if (!carried) {
             if (rec) {
                 if (lane == 0) P.ncert = 0;
+                if (lane < 27) P.supi[lane] = cert_sup(P.sup, lane);
                 __syncwarp();
             }
             // near-first rings for cells clipped from a list; a warm-started cell of the
@@ -1744,7 +1920,23 @@ __device__ __forceinline__ bool process_cell(Poly<R, C>& P, const ClipParams& cp
             // below clips every seed that cuts whatever the order
             if (MODE == MODE_FULL && !(warm && cp.pass == 3))
                 done = ring_walk(P, cp, cc, b, zprev, lane, bad, st);
-            if (done) done = traverse<R, C, MODE>(P, cp, cc, b, lane, bad, st);
+            if (done) {
+                // MODE_FULL: usually nothing cuts any more; where something does, the
+                // pyramid walk clips by it (in its own order)
+                const int wr = window_walk(P, cp, cc, b, lane, bad, st);
+                if (MODE == MODE_CERTIFY) {
+                    if (wr == WALK_STOP) done = false;
+                } else if (wr == WALK_STOP) {
+                    st &= ~(uint32_t)CS_UNCERTIFIED;
+                }
+                if (wr == WALK_OTHER || (MODE == MODE_FULL && wr == WALK_STOP)) {
+                    if (rec) {
+                        if (lane == 0) P.ncert = 0;
+                        __syncwarp();
+                    }
+                    done = traverse<R, C, MODE>(P, cp, cc, b, lane, bad, st);
+                }
+            }
             if (done && rec) {
                 __syncwarp();
                 ncert = P.ncert;
