@@ -62,6 +62,44 @@ struct Cap {
 using CapS = Cap<64, 128, 256>;
 using CapL = Cap<96, 192, 512>;
 
+// The cell's own seed in grid-local form: integer grid cell and FP32 offset from the
+// grid cell's corner (units of a), psi/a^2 split into two floats (hi + lo).
+struct SeedRef {
+    int c[3];
+    float off[3];
+    uint32_t io[3];
+    float phi, plo;
+};
+
+// Frame of the FP32 polytope of one cell: origin z (units of a, relative to the
+// seed), snapped to multiples of 2^-12 grid cells so that z is exact in FP64 and
+// nearly so in FP32.
+struct Frame {
+    float z[3];    // z in FP32
+    double zd[3];  // z in FP64
+};
+
+// Current bounds of the polytope (seed-relative coordinates, units of a): the centre c of
+// its bounding box, the radius Rc of the ball around c holding every vertex, and Mv = max
+// over the vertices of 1/2 |v|^2.
+struct Bounds {
+    float zf[3];  // frame origin of the polytope's vertices (relative to the seed)
+    float c[3];
+    float Rc;
+    float Mv;
+    float cabs[3];  // c in absolute coordinates, wrapped into the box
+    float yabs[3];  // the seed in absolute coordinates
+    float psi_i;    // psi_i / a^2 (hi part)
+};
+
+struct CellCtx {
+    int64_t i;
+    Pos4 yi;      // FP64 seed (FP64 planes)
+    double psii;  // FP64 psi_i
+    SeedRef si;   // grid-local seed (FP32 planes)
+    Frame fr;     // frame of the polytope (the seed itself for FP64 cells)
+};
+
 template <typename R, class C>
 struct Poly {
     V4<R> pl[C::MP];          // plane p.n <= w (frame coordinates)
@@ -90,12 +128,26 @@ struct Poly {
     };
     float sup[27];            // support max_v v.u over the 26 stencil directions u
     float supi[27];           // the same inflated for the certificate (cert_sup)
+    CellCtx cc;               // the cell: seed, psi, frame
+    Bounds b;                 // bounds of the polytope (poly_bounds)
+    float zprev[3];           // previous centroid, relative to the seed
+    float cen[3];             // centroid (integrate), relative to the seed
     int np, nt;
     int ncert;                // seeds recorded for the cell's certificate (-1: too many)
 #ifdef SDOT_COUNTERS
     uint32_t wc[8];           // work counters of the current cell (diagnostic builds)
 #endif
 };
+
+// A block's polytopes, one or two a warp, fill its dynamic shared memory. The routines
+// take a polytope's slot, not its address: through the array the compiler knows that every
+// access is to shared memory. What is the same for a warp (the cell's context, its
+// bounds) is kept there too, once, and not in every lane's stack frame.
+extern __shared__ __align__(16) unsigned char g_polytopes[];
+template <typename R, class C>
+__device__ __forceinline__ Poly<R, C>& poly_at(int slot) {
+    return reinterpret_cast<Poly<R, C>*>(g_polytopes)[slot];
+}
 
 // Work counters, compiled in only with -DSDOT_COUNTERS (diagnostic builds). The
 // count argument is evaluated by lane 0 only, so it must not contain a warp vote.
@@ -221,7 +273,9 @@ __device__ __forceinline__ void set_vert(Poly<R, C>& P, int s, const V3<R>& v) {
 // The periodic box around the seed: the bisectors of the cell's own images at
 // +-Lt e_a, written relative to the frame origin z (zero: the seed itself).
 template <typename R, class C>
-__device__ void poly_init(Poly<R, C>& P, const ClipParams& cp, const float* z, int lane) {
+__device__ __noinline__ void poly_init(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const float* z = P.cc.fr.z;
     if (lane < 6) {
         int ax = lane >> 1;
         R s = (lane & 1) ? R(-1) : R(1);
@@ -272,7 +326,8 @@ __device__ __forceinline__ V3<R> vertex_of(const Poly<R, C>& P, uint32_t t, R dt
 
 // drop planes no vertex references any more; returns the number of planes left
 template <typename R, class C>
-__device__ __noinline__ int poly_gc(Poly<R, C>& P, int lane) {
+__device__ __noinline__ int poly_gc(int slot, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
     constexpr int NW = (C::MP + 31) / 32;
     uint32_t used[NW];
 #pragma unroll
@@ -346,7 +401,7 @@ __device__ __noinline__ int poly_gc(Poly<R, C>& P, int lane) {
     return nn;
 }
 
-enum { CLIP_NONE = 0, CLIP_CUT = 1, CLIP_EMPTY = 2, CLIP_CAP = 3 };
+enum { CLIP_NONE = 0, CLIP_CUT = 1, CLIP_EMPTY = 2, CLIP_CAP = 3, CLIP_BAD = 4 };
 
 // relative tolerance of the vertex classification: a vertex counts as outside only
 // when it is beyond the plane by more than this fraction of the terms involved, so
@@ -364,8 +419,8 @@ __device__ __forceinline__ bool beyond(const V3<R>& v, const V4<R>& pn, R plen, 
 
 // Does the plane cut the polytope (some vertex strictly beyond it)? Warp-uniform.
 template <typename R, class C>
-__device__ __noinline__ bool poly_cut_by(const Poly<R, C>& P, const V4<R>& pn, R plen,
-                                         int lane) {
+__device__ __noinline__ bool poly_cut_by(int slot, V4<R> pn, R plen, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
     bool o = false;
     for (int q = lane; q < P.nt; q += 32) {
         R sd;
@@ -374,7 +429,8 @@ __device__ __noinline__ bool poly_cut_by(const Poly<R, C>& P, const V4<R>& pn, R
     return __any_sync(FULLMASK, o);
 }
 
-// Clip by p.n <= w (tag j). Non-finite geometry sets bad. Warp-uniform.
+// Clip by p.n <= w (tag j). Returns CLIP_*; CLIP_CUT with CLIP_BAD added when the geometry
+// is not finite. Warp-uniform.
 //
 // Bound by the instructions one warp issues, so both inner parts give every lane work:
 //  - an edge x -> y of a removed dual triangle lies on the boundary when no removed
@@ -386,8 +442,8 @@ __device__ __noinline__ bool poly_cut_by(const Poly<R, C>& P, const V4<R>& pn, R
 // First diagram of a 97^3 box, mixed: 219 -> 182 ms; FP64 evaluations of a 45^3 box, whose
 // vertex arithmetic fills the FP64 pipe: 31.6 -> 24.1 ms; the mesh deposit 92.7 -> 54.2 ms.
 template <typename R, class C>
-__device__ __noinline__ int poly_clip(Poly<R, C>& P, const V4<R>& pn, R plen, int32_t j,
-                                      int lane, bool& bad) {
+__device__ __noinline__ int poly_clip(int slot, V4<R> pn, R plen, int32_t j, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
     constexpr int SL = C::SL, NW = C::NW;
     static_assert(sizeof(P.adj) <= 3 * C::MNEW * sizeof(R), "the table shares the new vertices");
     const int nt = P.nt;
@@ -413,7 +469,7 @@ __device__ __noinline__ int poly_clip(Poly<R, C>& P, const V4<R>& pn, R plen, in
     if (nrem == nt) return CLIP_EMPTY;
     if (nrem > C::MREM) return CLIP_CAP;
     if (P.np >= C::MP) {
-        if (poly_gc(P, lane) >= C::MP) return CLIP_CAP;
+        if (poly_gc<R, C>(slot, lane) >= C::MP) return CLIP_CAP;
     }
     const uint32_t ps = (uint32_t)P.np;
     const uint32_t below = lanes_below(lane);
@@ -555,9 +611,9 @@ __device__ __noinline__ int poly_clip(Poly<R, C>& P, const V4<R>& pn, R plen, in
         P.np = ps + 1;
         P.nt = nkept + nnew;
     }
-    if (__any_sync(FULLMASK, lbad)) bad = true;
+    lbad = __any_sync(FULLMASK, lbad);
     __syncwarp();
-    return CLIP_CUT;
+    return lbad ? CLIP_CUT | CLIP_BAD : CLIP_CUT;
 }
 
 // is seed j already one of the polytope's planes? (warp-uniform j)
@@ -568,67 +624,15 @@ __device__ __forceinline__ bool has_plane(const Poly<R, C>& P, int32_t j, int la
     return __any_sync(FULLMASK, dup);
 }
 
-// The cell's own seed in grid-local form: integer grid cell and FP32 offset from the
-// grid cell's corner (units of a), psi/a^2 split into two floats (hi + lo).
-struct SeedRef {
-    int c[3];
-    float off[3];
-    uint32_t io[3];
-    float phi, plo;
-};
-
-__device__ __forceinline__ SeedRef load_seed(const ClipParams& cp, int64_t i) {
-    SeedRef r;
-    float4 p = cp.posf[i];
-    int lc = cp.leafc[i];
-    r.c[0] = lc & 1023;
-    r.c[1] = (lc >> 10) & 1023;
-    r.c[2] = (lc >> 20) & 1023;
-    r.off[0] = p.x;
-    r.off[1] = p.y;
-    r.off[2] = p.z;
-    r.phi = p.w;
-    r.plo = cp.pslo[i];
-    uint4 q = cp.ioff[i];
-    r.io[0] = q.x;
-    r.io[1] = q.y;
-    r.io[2] = q.z;
-    return r;
-}
-
-// Frame of the FP32 polytope of one cell: origin z (units of a, relative to the
-// seed), snapped to multiples of 2^-12 grid cells so that z is exact in FP64 and
-// nearly so in FP32.
-struct Frame {
-    float z[3];    // z in FP32
-    double zd[3];  // z in FP64
-};
-
-__device__ __forceinline__ Frame make_frame(const ClipParams& cp, const float* zwant) {
-    Frame f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        float za = zwant[a];
-        if (!isfinite(za)) za = 0.f;
-        za = fminf(fmaxf(za, -cp.halfLt[a]), cp.halfLt[a]);
-        // snapped to a multiple of q = ht / 4096 (the nearest one up to FP32 rounding of
-        // the quotient; any multiple serves, the choice is deterministic)
-        const double q = (double)cp.ht[a] * (1.0 / 4096.0);
-        f.zd[a] = (double)llrintf(za * (4096.f / cp.ht[a])) * q;
-        f.z[a] = (float)f.zd[a];
-    }
-    return f;
-}
-
-// the frame at the seed itself (FP64 cells)
-__device__ __forceinline__ Frame seed_frame() {
-    Frame f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        f.z[a] = 0.f;
-        f.zd[a] = 0.0;
-    }
-    return f;
+__device__ __forceinline__ void frame_axis(const ClipParams& cp, float za, int a, Frame& f) {
+    if (!isfinite(za)) za = 0.f;
+    za = fminf(fmaxf(za, -cp.halfLt[a]), cp.halfLt[a]);
+    // snapped to a multiple of q = ht / 4096 (the nearest one up to FP32 rounding of
+    // the quotient; any multiple serves, the choice is deterministic)
+    const double q = (double)cp.ht[a] * (1.0 / 4096.0);
+    const double zd = (double)llrintf(za * (4096.f / cp.ht[a])) * q;
+    f.zd[a] = zd;
+    f.z[a] = (float)zd;
 }
 
 // plane of neighbour j for cell i, built in FP64 (normalised units, seed frame)
@@ -706,20 +710,6 @@ __device__ __forceinline__ void plane_f32(const ClipParams& cp, const SeedRef& s
     w = 0.5f * (nx * nx + ny * ny + nz * nz) + ((si.phi - pj.w) + (si.plo - cp.pslo[j]));
 }
 
-// Current bounds of the polytope (seed-relative coordinates, units of a): box
-// [bmin, bmax], its centre c, the radius Rc of the ball around c holding every
-// vertex, and Mv = max over the vertices of 1/2 |v|^2.
-struct Bounds {
-    float zf[3];  // frame origin of the polytope's vertices (relative to the seed)
-    float bmin[3], bmax[3];
-    float c[3];
-    float Rc;
-    float Mv;
-    float cabs[3];  // c in absolute coordinates, wrapped into the box
-    float yabs[3];  // the seed in absolute coordinates
-    float psi_i;    // psi_i / a^2 (hi part)
-};
-
 // order-preserving map of a float onto uint32, so a warp max runs on integers
 __device__ __forceinline__ uint32_t f2ord(float f) {
     const uint32_t u = __float_as_uint(f);
@@ -752,9 +742,9 @@ __device__ __forceinline__ float wrap_box(float x, float Lt) {
 // direction k (lane 13, the zero direction, takes |v|^2) and scans every vertex from
 // shared memory: one loop, no reductions for the 26 directions.
 template <typename R, class C>
-__device__ __noinline__ void poly_bounds(const Poly<R, C>& P, const ClipParams& cp, Bounds& b,
-                                         int lane) {
-    Poly<R, C>& Pm = const_cast<Poly<R, C>&>(P);
+__device__ __noinline__ void poly_bounds(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    Bounds& b = P.b;
     const float ux = (float)(lane % 3 - 1), uy = (float)((lane / 3) % 3 - 1),
                 uz = (float)(lane / 9 - 1);
     const float w2 = lane == 13 ? 1.f : 0.f;
@@ -767,31 +757,31 @@ __device__ __noinline__ void poly_bounds(const Poly<R, C>& P, const ClipParams& 
         const float d = fmaf(ux, x, fmaf(uy, y, uz * z));
         h = fmaxf(h, fmaf(w2, fmaf(x, x, fmaf(y, y, z * z)), d));
     }
-    if (lane < 27) Pm.sup[lane] = h;
+    if (lane < 27) P.sup[lane] = h;
     __syncwarp();
     // +x 14, -x 12, +y 16, -y 10, +z 22, -z 4
-    const int ip[3] = {14, 16, 22}, in[3] = {12, 10, 4};
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        b.bmax[a] = P.sup[ip[a]];
-        b.bmin[a] = -P.sup[in[a]];
-        b.c[a] = 0.5f * (b.bmin[a] + b.bmax[a]);
-    }
-    b.Mv = 0.5f * P.sup[13] * 1.0001f + 1e-6f;
-    __syncwarp();
-    if (lane == 0) Pm.sup[13] = 0.f;  // the zero direction (never used by the prefilter)
+    const float cx = 0.5f * (P.sup[14] - P.sup[12]), cy = 0.5f * (P.sup[16] - P.sup[10]),
+                cz = 0.5f * (P.sup[22] - P.sup[4]);
+    const float Mv = 0.5f * P.sup[13] * 1.0001f + 1e-6f;
     float r2 = 0.f;
 #pragma unroll 1
     for (int s = lane; s < nt; s += 32) {
-        const float dx = ((float)P.vx[s] + z0) - b.c[0];
-        const float dy = ((float)P.vy[s] + z1) - b.c[1];
-        const float dz = ((float)P.vz[s] + z2) - b.c[2];
+        const float dx = ((float)P.vx[s] + z0) - cx;
+        const float dy = ((float)P.vy[s] + z1) - cy;
+        const float dz = ((float)P.vz[s] + z2) - cz;
         r2 = fmaxf(r2, dx * dx + dy * dy + dz * dz);
     }
     r2 = warp_max(r2);
-    b.Rc = sqrtf(r2) * 1.0001f + 1e-5f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) b.cabs[a] = wrap_box(b.yabs[a] + b.c[a], cp.Lt[a]);
+    if (lane < 3) {  // one axis a lane
+        const float c = lane == 0 ? cx : (lane == 1 ? cy : cz);
+        b.c[lane] = c;
+        b.cabs[lane] = wrap_box(b.yabs[lane] + c, cp.Lt[lane]);
+    }
+    if (lane == 0) {
+        b.Mv = Mv;
+        b.Rc = sqrtf(r2) * 1.0001f + 1e-5f;
+        P.sup[13] = 0.f;  // the zero direction (never used by the prefilter)
+    }
     __syncwarp();
 }
 
@@ -920,15 +910,7 @@ __device__ __forceinline__ float cert_sup(const float* sup, int k) {
 }
 
 enum { MODE_CERTIFY = 0, MODE_FULL = 1 };
-enum { LEAF_OK = 0, LEAF_STOP = 1 };
-
-struct CellCtx {
-    int64_t i;
-    Pos4 yi;      // FP64 seed (FP64 planes)
-    double psii;  // FP64 psi_i
-    SeedRef si;   // grid-local seed (FP32 planes)
-    Frame fr;     // frame of the polytope (the seed itself for FP64 cells)
-};
+enum : uint32_t { STOP_BITS = 0xff, WALK_BAD = 0x100 };  // results of the walks
 
 // exact plane of seed j in the polytope's frame (per lane)
 template <typename R>
@@ -980,8 +962,9 @@ __device__ __forceinline__ bool among(const int32_t (&pj)[NW], int32_t j) {
 // Per lane: can the FP32 plane (seed frame) reach a vertex? Conservative like the
 // prefilter: it may differ from the exact plane by the margin.
 template <typename R, class C>
-__device__ __noinline__ bool reaches_vertex(const Poly<R, C>& P, const Bounds& b, float nx, float ny,
-                                            float nz, float w) {
+__device__ __noinline__ bool reaches_vertex(int slot, float nx, float ny, float nz, float w) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Bounds& b = P.b;
     const float z0 = b.zf[0], z1 = b.zf[1], z2 = b.zf[2];
     float h = -INFINITY;
 #pragma unroll 1
@@ -1001,11 +984,16 @@ constexpr int VERTEX_TEST_MIN = 7;
 // The seeds of every lane's two runs [s0, s0 + n0) and [s1, s1 + n1) of the sorted order,
 // spread evenly over the lanes: each seed passes the conservative prefilter in its lane,
 // the survivors are checked exactly one by one (warp-uniform). CERTIFY stops at the first
-// seed that cuts; FULL clips it. Returns LEAF_STOP when the cell's processing must stop.
+// seed that cuts; FULL clips it. Returns status bits: CS_UNCERTIFIED, CS_EMPTY or
+// CS_CAPACITY when the cell's processing must stop (STOP_BITS), WALK_BAD for geometry that
+// is not finite.
 template <typename R, class C, int MODE>
-__device__ __noinline__ int process_seeds(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                          Bounds& b, int32_t s0, int n0, int32_t s1, int n1,
-                                          int lane, bool& bad, uint32_t& st) {
+__device__ __noinline__ uint32_t process_seeds(int slot, const ClipParams& cp, int32_t s0, int n0,
+                                               int32_t s1, int n1, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const CellCtx& cc = P.cc;
+    const Bounds& b = P.b;
+    uint32_t bad = 0;
     const int n = n0 + n1;
     int incl = n;
     for (int o = 1; o < 32; o <<= 1) {
@@ -1071,7 +1059,7 @@ __device__ __noinline__ int process_seeds(Poly<R, C>& P, const ClipParams& cp, c
             __syncwarp();
         }
         if (__popc(cm) >= VERTEX_TEST_MIN) {
-            cand = ((cm >> lane) & 1u) && reaches_vertex(P, b, nx, ny, nz, w);
+            cand = ((cm >> lane) & 1u) && reaches_vertex<R, C>(slot, nx, ny, nz, w);
             cm = __ballot_sync(FULLMASK, cand);
         }
         if (!cm) continue;
@@ -1087,39 +1075,30 @@ __device__ __noinline__ int process_seeds(Poly<R, C>& P, const ClipParams& cp, c
             const V4<R> pn = shfl_plane(pl, src);
             const R plen = __shfl_sync(FULLMASK, len, src);
             if (MODE == MODE_CERTIFY) {
-                if (poly_cut_by(P, pn, plen, lane)) {
-                    st |= CS_UNCERTIFIED;
-                    return LEAF_STOP;
-                }
+                if (poly_cut_by<R, C>(slot, pn, plen, lane)) return CS_UNCERTIFIED;
                 continue;
             }
             const int32_t j = __shfl_sync(FULLMASK, s, src);
-            const int rc = poly_clip(P, pn, plen, j, lane, bad);
-            if (rc == CLIP_EMPTY) {
-                st |= CS_EMPTY;
-                return LEAF_STOP;
-            }
-            if (rc == CLIP_CAP) {
-                st |= CS_CAPACITY | CS_CAP_POLY;
-                return LEAF_STOP;
-            }
-            cut |= rc == CLIP_CUT;
+            const int rc = poly_clip<R, C>(slot, pn, plen, j, lane);
+            if (rc == CLIP_EMPTY) return CS_EMPTY | bad;
+            if (rc == CLIP_CAP) return CS_CAPACITY | CS_CAP_POLY | bad;
+            if (rc & CLIP_BAD) bad = WALK_BAD;
+            cut |= rc != CLIP_NONE;
         }
         // the bounds of this round's start stay valid (larger) for its later seeds, whose
         // exact test decides; the next round starts from the smaller polytope
         if (MODE == MODE_FULL && cut) {
-            poly_bounds(P, cp, b, lane);
+            poly_bounds<R, C>(slot, cp, lane);
             load_planes(P, pj, lane);
         }
     }
-    return LEAF_OK;
+    return bad;
 }
 
 // the seeds of up to 32 grid cells (leaf < 0: none)
 template <typename R, class C, int MODE>
-__device__ __forceinline__ int process_leaves(Poly<R, C>& P, const ClipParams& cp,
-                                              const CellCtx& cc, Bounds& b, int64_t leaf, int lane,
-                                              bool& bad, uint32_t& st) {
+__device__ __forceinline__ uint32_t process_leaves(int slot, const ClipParams& cp, int64_t leaf,
+                                                   int lane) {
     int32_t sb = 0;
     int n = 0;
     if (leaf >= 0) {
@@ -1129,22 +1108,23 @@ __device__ __forceinline__ int process_leaves(Poly<R, C>& P, const ClipParams& c
 #ifdef SDOT_COUNTERS
     {
         const uint32_t nleaf = __popc(__ballot_sync(FULLMASK, leaf >= 0));
-        WCOUNT(P, 3, nleaf);
+        WCOUNT((poly_at<R, C>(slot)), 3, nleaf);
     }
 #endif
-    return process_seeds<R, C, MODE>(P, cp, cc, b, sb, n, sb + n, 0, lane, bad, st);
+    return process_seeds<R, C, MODE>(slot, cp, sb, n, sb + n, 0, lane);
 }
 
 // Near-first pass for re-queued cells: the grid cells in Chebyshev rings around the
 // grid cell of the previous centroid, so the polytope is small before the walk starts.
 template <typename R, class C>
-__device__ __noinline__ bool ring_walk(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                       Bounds& b, const float* zprev, int lane, bool& bad,
-                                       uint32_t& st) {
+__device__ __noinline__ uint32_t ring_walk(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Bounds& b = P.b;
+    uint32_t out = 0;
     int ca[3];
     float hmin = 1e30f;
     for (int a = 0; a < 3; a++) {
-        float za = fmodf(b.yabs[a] + zprev[a], cp.Lt[a]);
+        float za = fmodf(b.yabs[a] + P.zprev[a], cp.Lt[a]);
         if (za < 0.f) za += cp.Lt[a];
         int c = (int)floorf(za / cp.ht[a]);
         ca[a] = c < 0 ? 0 : (c >= cp.G[a] ? cp.G[a] - 1 : c);
@@ -1175,15 +1155,15 @@ __device__ __noinline__ bool ring_walk(Poly<R, C>& P, const ClipParams& cp, cons
                     leaf = ((int64_t)c[2] * cp.G[1] + c[1]) * cp.G[0] + c[0];
                 }
             }
-            if (process_leaves<R, C, MODE_FULL>(P, cp, cc, b, leaf, lane, bad, st) == LEAF_STOP)
-                return false;
+            out |= process_leaves<R, C, MODE_FULL>(slot, cp, leaf, lane);
+            if (out & STOP_BITS) return out;
         }
     }
-    return true;
+    return out;
 }
 
-// Walk the pyramid. MODE_CERTIFY: return false as soon as a seed cuts the polytope.
-// MODE_FULL: clip every such seed. Returns true when the walk completed. A stack entry
+// Walk the pyramid. MODE_CERTIFY: stop as soon as a seed cuts the polytope. MODE_FULL: clip
+// every such seed. Returns status bits as process_seeds does. A stack entry
 // is a node to expand: level << 27 | Z << 18 | Y << 9 | X (levels >= 1 have at most
 // 256 nodes per axis); its children are the up to 4 x 4 x 4 nodes one level down. The
 // root is the virtual node (nlev, 0, 0, 0) whose children are the top level.
@@ -1203,8 +1183,10 @@ __device__ __forceinline__ WalkBall walk_ball(const Bounds& b, bool rec) {
 }
 
 template <typename R, class C, int MODE>
-__device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                      Bounds& b, int lane, bool& bad, uint32_t& st) {
+__device__ __noinline__ uint32_t traverse(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Bounds& b = P.b;
+    uint32_t out = 0;
     if (lane == 0) P.stack[0] = pack_node(cp.pyr.nlev, 0, 0, 0);
     int sp = 1;
     const float Lt[3] = {cp.Lt[0], cp.Lt[1], cp.Lt[2]};
@@ -1234,10 +1216,7 @@ __device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const
             if (sm == 0) continue;
             if (cl > 0) {
                 const int n = __popc(sm);
-                if (sp + n > C::STK) {
-                    st |= CS_CAPACITY | CS_CAP_STACK;
-                    return false;
-                }
+                if (sp + n > C::STK) return out | CS_CAPACITY | CS_CAP_STACK;
                 if (surv) P.stack[sp + __popc(sm & lanes_below(lane))] = pack_node(cl, cx, cy, cz);
                 sp += n;
                 __syncwarp();
@@ -1245,12 +1224,12 @@ __device__ __noinline__ bool traverse(Poly<R, C>& P, const ClipParams& cp, const
             }
             // surviving grid cells: their seeds
             const int64_t leaf = surv ? ((int64_t)cz * cp.G[1] + cy) * cp.G[0] + cx : -1;
-            if (process_leaves<R, C, MODE>(P, cp, cc, b, leaf, lane, bad, st) == LEAF_STOP)
-                return false;
+            out |= process_leaves<R, C, MODE>(slot, cp, leaf, lane);
+            if (out & STOP_BITS) return out;
             if (MODE == MODE_FULL) wb = walk_ball(b, false);  // a clip may have shrunk the polytope
         }
     }
-    return true;
+    return out;
 }
 
 // The certifying walk by a window. The pyramid is walked down to level 1 only (nodes of
@@ -1271,8 +1250,9 @@ enum { WALK_DONE = 0, WALK_STOP = 1, WALK_OTHER = 2 };
 constexpr int WINDOW_CELLS = 1000;
 
 template <typename R, class C>
-__device__ __noinline__ int window_walk(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                        Bounds& b, int lane, bool& bad, uint32_t& st) {
+__device__ __noinline__ int window_walk(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Bounds& b = P.b;
     if (cp.pyr.nlev < 2) return WALK_OTHER;
     if (lane == 0) P.stack[0] = pack_node(cp.pyr.nlev, 0, 0, 0);
     int sp = 1;
@@ -1364,20 +1344,22 @@ __device__ __noinline__ int window_walk(Poly<R, C>& P, const ClipParams& cp, con
                 }
             }
         }
-        if (process_seeds<R, C, MODE_CERTIFY>(P, cp, cc, b, s0, n0, s1, n1, lane, bad, st) ==
-            LEAF_STOP)
-            return WALK_STOP;
+        if (process_seeds<R, C, MODE_CERTIFY>(slot, cp, s0, n0, s1, n1, lane)) return WALK_STOP;
     }
     return WALK_DONE;
 }
 
-// Integrate the polytope and write the outputs of cell i; cen receives the centroid
-// relative to the seed (units of a, every lane) and the return value says whether it
-// is valid (positive finite volume).
+// Integrate the polytope and write the outputs of its cell; P.cen receives the centroid
+// relative to the seed (units of a). Returns status bits: CS_CAPACITY, CS_INCONSISTENT for a
+// failed check, INT_VALID when the centroid is valid (positive finite volume).
+enum : uint32_t { INT_VALID = 0x100 };
 template <typename R, class C>
-__device__ __noinline__ bool integrate(Poly<R, C>& P, const ClipParams& cp, const Frame& fr,
-                                       int64_t i, int lane, bool& bad, uint32_t& st,
-                                       float* cen) {
+__device__ __noinline__ uint32_t integrate(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Frame& fr = P.cc.fr;
+    const int64_t i = P.cc.i;
+    bool bad = false;
+    uint32_t st = 0;
     // volume and first moment: summed per face in R, the face totals in FP64; the
     // surface closure check and the facet areas in R
     double vol6 = 0, mx = 0, my = 0, mz = 0;
@@ -1622,6 +1604,7 @@ __device__ __noinline__ bool integrate(Poly<R, C>& P, const ClipParams& cp, cons
     st = __reduce_or_sync(FULLMASK, st);
     const double mm[3] = {mx * (1.0 / 24.0), my * (1.0 / 24.0), mz * (1.0 / 24.0)};
     const bool valid = vol > 0.0 && isfinite(vol);
+    float cen[3] = {0.f, 0.f, 0.f};
     if (valid) {
         // the centroid is kept in FP32 (frame anchor): one FP32 division per axis
         const float fv = (float)vol;
@@ -1637,19 +1620,19 @@ __device__ __noinline__ bool integrate(Poly<R, C>& P, const ClipParams& cp, cons
         cp.fcnt[i] = total > FCAP ? FCAP : total;
         cp.topo_n[i] = (uint8_t)(tok && valid ? nt : 0);
         if (valid) {
-            cp.anchor[3 * i + 0] = cen[0];
-            cp.anchor[3 * i + 1] = cen[1];
-            cp.anchor[3 * i + 2] = cen[2];
+            for (int a = 0; a < 3; a++) cp.anchor[3 * i + a] = P.cen[a] = cen[a];
         }
     }
-    return valid;
+    __syncwarp();
+    return st | (bad ? CS_INCONSISTENT : 0u) | (valid ? INT_VALID : 0u);
 }
 
 // The cell must stay inside the minimum-image range of every other seed: radius R0 of
 // the polytope about the seed against half the box.
 template <typename R, class C>
-__device__ __noinline__ bool cell_too_large(const Poly<R, C>& P, const CellCtx& cc,
-                                            float psimax_glob, float halfLmin, int lane) {
+__device__ __noinline__ bool cell_too_large(int slot, float psimax_glob, float halfLmin, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const CellCtx& cc = P.cc;
     float r2 = 0.f;
     for (int s = lane; s < P.nt; s += 32) {
         const float dx = (float)P.vx[s] + cc.fr.z[0], dy = (float)P.vy[s] + cc.fr.z[1],
@@ -1668,10 +1651,14 @@ constexpr float REFRAME_DIST = 0.5f;
 
 // Clip by a list of seeds (warp-uniform count): each lane builds one plane, then the
 // warp clips by them in order; entries out of range and seeds already among the
-// planes are skipped.
+// planes are skipped. Returns CLIP_NONE, CLIP_EMPTY or CLIP_CAP, with CLIP_BAD added where
+// the geometry is not finite.
 template <typename R, class C>
-__device__ __noinline__ int clip_list(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                      const int32_t* list, int n, int lane, bool& bad) {
+__device__ __noinline__ int clip_list(int slot, const ClipParams& cp, const int32_t* list, int n,
+                                      int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const CellCtx& cc = P.cc;
+    int bad = 0;
     for (int t0 = 0; t0 < n; t0 += 32) {
         const int t = t0 + lane;
         V4<R> pl;
@@ -1690,11 +1677,12 @@ __device__ __noinline__ int clip_list(Poly<R, C>& P, const ClipParams& cp, const
             const V4<R> pn = shfl_plane(pl, u);
             const R plen = __shfl_sync(FULLMASK, len, u);
             if (has_plane(P, ju, lane)) continue;
-            const int rc = poly_clip(P, pn, plen, ju, lane, bad);
-            if (rc == CLIP_EMPTY || rc == CLIP_CAP) return rc;
+            const int rc = poly_clip<R, C>(slot, pn, plen, ju, lane);
+            if (rc == CLIP_EMPTY || rc == CLIP_CAP) return rc | bad;
+            bad |= rc & CLIP_BAD;
         }
     }
-    return CLIP_NONE;
+    return CLIP_NONE | bad;
 }
 
 // Warm start from the cell's stored topology: the planes of its previous facets (and
@@ -1706,10 +1694,11 @@ __device__ __noinline__ int clip_list(Poly<R, C>& P, const ClipParams& cp, const
 // one is more than half a box from its seed, which the size check reports.) Returns
 // false when the check fails; the caller then clips from the box.
 template <typename R, class C>
-__device__ __noinline__ bool topo_init(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                       int nf, int nt, int lane) {
+__device__ __noinline__ bool topo_init(int slot, const ClipParams& cp, int nf, int nt, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const CellCtx& cc = P.cc;
     if (6 + nf > C::MP || nt > C::MT || nt > TOPO || nt < 4) return false;
-    poly_init(P, cp, cc.fr.z, lane);  // the box planes in slots 0..5
+    poly_init<R, C>(slot, cp, lane);  // the box planes in slots 0..5
     bool ok = true;
 #pragma unroll 1
     for (int k = lane; k < nf; k += 32) {
@@ -1775,8 +1764,11 @@ __device__ __forceinline__ float top_psimax(const ClipParams& cp, int lane) {
 // it still certifies the cell (see CERT_EPS above). The reserves it used are then written
 // back, less the change of psi differences of this evaluation.
 template <typename R, class C>
-__device__ __noinline__ bool cert_check(Poly<R, C>& P, const ClipParams& cp, const CellCtx& cc,
-                                        const Bounds& b, int64_t i, int nc, int lane) {
+__device__ __noinline__ bool cert_check(int slot, const ClipParams& cp, int nc, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const CellCtx& cc = P.cc;
+    const Bounds& b = P.b;
+    const int64_t i = cc.i;
     const float* cf = cp.cert_f + i * CERT_F;
     const float c0 = cf[0], c1 = cf[1], c2 = cf[2], Rt = cf[3], Mr = cf[4], Wr = cf[5];
     const float hi = ord2f(cp.cert_dpsi[0]), lo = ord2f(cp.cert_dpsi[1]);
@@ -1816,7 +1808,7 @@ __device__ __noinline__ bool cert_check(Poly<R, C>& P, const ClipParams& cp, con
         m &= m - 1;
         const V4<R> pn = shfl_plane(pl, src);
         const R plen = __shfl_sync(FULLMASK, len, src);
-        if (poly_cut_by(P, pn, plen, lane)) return false;
+        if (poly_cut_by<R, C>(slot, pn, plen, lane)) return false;
     }
     if (lane == 0) {
         cp.cert_f[i * CERT_F + 4] = Mn;
@@ -1828,8 +1820,10 @@ __device__ __noinline__ bool cert_check(Poly<R, C>& P, const ClipParams& cp, con
 // Record the certificate of a certifying walk (bounds b before the walk, the seeds in
 // P.ftri); its count is set once the cell's outputs are known to be clean.
 template <typename R, class C>
-__device__ __noinline__ void cert_store(const Poly<R, C>& P, const ClipParams& cp, const Bounds& b,
-                                        int64_t i, int lane) {
+__device__ __noinline__ void cert_store(int slot, const ClipParams& cp, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    const Bounds& b = P.b;
+    const int64_t i = P.cc.i;
     if (lane < 27)
         cp.cert_s[i * CERT_S + lane] =
             lane == 13 ? (uint16_t)0 : __half_as_ushort(__float2half_ru(P.supi[lane]));
@@ -1846,155 +1840,202 @@ __device__ __noinline__ void cert_store(const Poly<R, C>& P, const ClipParams& c
     }
 }
 
-// One work item w of a clipping pass: cell worklist[w] (or w), clipped by its first
-// candidates, certified (pass 1) or walked (re-queue pass), integrated; outputs
-// written, the cell queued for the next pass where needed. BIG: the large-capacity
-// FP64 re-clip, after which no pass follows.
+// The cell's context: seed, psi, previous centroid, and the polytope's frame (FP32 cells:
+// at the previous centroid; FP64 cells: at the seed). One axis a lane.
+template <typename R, class C>
+__device__ __forceinline__ void load_cell(int slot, const ClipParams& cp, int64_t i, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    CellCtx& cc = P.cc;
+    __syncwarp();  // the last cell's reads are done
+    float z = lane < 3 ? cp.anchor[3 * i + lane] : 0.f;
+    if (!__all_sync(FULLMASK, isfinite(z))) z = 0.f;
+    if (lane < 3) {
+        const int c = (cp.leafc[i] >> (10 * lane)) & 1023;
+        const float off = reinterpret_cast<const float*>(cp.posf + i)[lane];
+        P.zprev[lane] = z;
+        cc.si.c[lane] = c;
+        cc.si.off[lane] = off;
+        cc.si.io[lane] = reinterpret_cast<const uint32_t*>(cp.ioff + i)[lane];
+        cc.fr.z[lane] = 0.f;
+        cc.fr.zd[lane] = 0.0;
+        if (sizeof(R) == 4) frame_axis(cp, z, lane, cc.fr);
+        P.b.zf[lane] = cc.fr.z[lane];
+        P.b.yabs[lane] = (float)c * cp.ht[lane] + off;
+    } else if (lane == 3) {
+        const float phi = cp.posf[i].w;
+        cc.si.phi = P.b.psi_i = phi;
+        cc.si.plo = cp.pslo[i];
+        cc.i = i;
+    } else if (lane == 4 && sizeof(R) == 8) {
+        cc.yi = cp.pos[i];
+        cc.psii = cp.psi[i];
+    }
+    __syncwarp();
+}
+
+// One work item w of a clipping pass for every warp of the block (act: the warp has one):
+// cell worklist[w] (or w), clipped by its first candidates, certified (pass 1) or walked
+// (re-queue pass), integrated; outputs written, the cell queued for the next pass where
+// needed. BIG: the large-capacity FP64 re-clip, after which no pass follows.
+//
+// The block's warps go through the phases together, a barrier between them. The whole of
+// it is several times the instruction cache; warps in different phases evicted each
+// other's code, and two thirds of every warp's time went to fetching instructions (stall
+// no_instruction 20 of 31 cycles per issue). With the context in shared memory, before and
+// after: first diagram 97^3 186 -> 132 ms, early Newton step 100^3 248 -> 121 ms, FP64 step
+// 45^3 22.0 -> 16.3 ms.
 template <typename R, class C, int MODE>
-__device__ __forceinline__ bool process_cell(Poly<R, C>& P, const ClipParams& cp, int64_t w,
+__device__ __forceinline__ bool process_cell(int slot, const ClipParams& cp, bool act, int64_t w,
                                              float psimax_glob, float halfLmin, int lane) {
     constexpr bool BIG = C::MP > CapS::MP;
-    CellCtx cc;
-    cc.i = cp.worklist ? cp.worklist[w] : w;
-    const int64_t i = cc.i;
-    cc.yi = cp.pos[i];
-    cc.psii = cp.psi[i];
-    cc.si = load_seed(cp, i);
-    bool bad = false;
+    Poly<R, C>& P = poly_at<R, C>(slot);
+    bool bad = false, warm = false;
     uint32_t st = 0;
-    float zprev[3] = {cp.anchor[3 * i], cp.anchor[3 * i + 1], cp.anchor[3 * i + 2]};
-    if (!(isfinite(zprev[0]) && isfinite(zprev[1]) && isfinite(zprev[2])))
-        zprev[0] = zprev[1] = zprev[2] = 0.f;
-    // FP32 cells: frame at the previous centroid; FP64 cells: at the seed
-    cc.fr = sizeof(R) == 4 ? make_frame(cp, zprev) : seed_frame();
-#ifdef SDOT_COUNTERS
-    if (lane < 8) P.wc[lane] = 0;
-    __syncwarp();
-    WCOUNT(P, 6, 1);
-#endif
+    int64_t i = 0;
+    int nprev = 0;
     // first candidates: the cell's facets in the previous diagram (its stored
     // topology when that still holds), then its k nearest seeds (every cell of the
     // first diagram, and any cell without facets)
-    int rc = CLIP_NONE;
-    const int nprev = cp.facets_valid ? min(cp.fcnt[i], FCAP) : 0;
-    const int ntopo = cp.facets_valid ? (int)cp.topo_n[i] : 0;
-    bool warm = false;
-    if (nprev > 0 && ntopo > 0) warm = topo_init(P, cp, cc, nprev, ntopo, lane);
-    if (!warm) {
-        poly_init(P, cp, cc.fr.z, lane);
-        if (nprev > 0) rc = clip_list(P, cp, cc, cp.fcol + i * FCAP, nprev, lane, bad);
-        if (nprev == 0 && rc == CLIP_NONE)
-            rc = clip_list(P, cp, cc, cp.knn + i * cp.k, cp.k, lane, bad);
+    if (act) {
+        i = cp.worklist ? cp.worklist[w] : w;
+        load_cell<R, C>(slot, cp, i, lane);
+#ifdef SDOT_COUNTERS
+        if (lane < 8) P.wc[lane] = 0;
+        __syncwarp();
+        WCOUNT(P, 6, 1);
+#endif
+        nprev = cp.facets_valid ? min(cp.fcnt[i], FCAP) : 0;
+        const int ntopo = cp.facets_valid ? (int)cp.topo_n[i] : 0;
+        if (nprev > 0 && ntopo > 0) warm = topo_init<R, C>(slot, cp, nprev, ntopo, lane);
     }
-    if (rc == CLIP_EMPTY) st |= CS_EMPTY;
-    if (rc == CLIP_CAP) st |= CS_CAPACITY | CS_CAP_POLY;
+    __syncthreads();
+    if (act && !warm) {
+        poly_init<R, C>(slot, cp, lane);
+        const int rc = nprev > 0
+                           ? clip_list<R, C>(slot, cp, cp.fcol + i * FCAP, nprev, lane)
+                           : clip_list<R, C>(slot, cp, cp.knn + i * cp.k, cp.k, lane);
+        bad = (rc & CLIP_BAD) != 0;
+        if ((rc & 3) == CLIP_EMPTY) st |= CS_EMPTY;
+        if ((rc & 3) == CLIP_CAP) st |= CS_CAPACITY | CS_CAP_POLY;
+    }
+    __syncthreads();
     // a certifying first pass carries the cell's security certificate between
     // evaluations (see CERT_EPS): used when it still holds, recorded after a walk
     const bool rec = MODE == MODE_CERTIFY && cp.pass == 1 && cp.cert_use;
     // the FP64 re-clip of a cell the FP32 check sent there uses the certificate the
     // first pass kept for it, checked against the FP64 polytope
     const bool use3 = MODE == MODE_FULL && !BIG && cp.pass == 3 && cp.cert_use;
-    bool carried = false, stored = false, reframed = false;
+    bool carried = false, stored = false, queued = false;
     int ncert = -1;
-    if (!st) {
-        Bounds b;
-        for (int a = 0; a < 3; a++) {
-            b.yabs[a] = (float)cc.si.c[a] * cp.ht[a] + cc.si.off[a];
-            b.zf[a] = cc.fr.z[a];
-        }
-        b.psi_i = cc.si.phi;
-        poly_bounds(P, cp, b, lane);
+    if (act && !st) {
+        poly_bounds<R, C>(slot, cp, lane);
         if ((rec || use3) && warm) {
             const int nc = cp.cert_n[i];
-            if (nc != 0xff) carried = cert_check(P, cp, cc, b, i, nc, lane);
+            if (nc != 0xff) carried = cert_check<R, C>(slot, cp, nc, lane);
         }
-        bool done = true;
-        if (!carried) {
+        if (!carried && rec) {
+            if (lane == 0) P.ncert = 0;
+            if (lane < 27) P.supi[lane] = cert_sup(P.sup, lane);
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    // near-first rings for cells clipped from a list; a warm-started cell of the
+    // FP64 re-clip already holds the FP32 pass's polytope, and the pyramid walk
+    // below clips every seed that cuts whatever the order
+    if (MODE == MODE_FULL) {
+        if (act && !st && !carried && !(warm && cp.pass == 3)) {
+            const uint32_t out = ring_walk<R, C>(slot, cp, lane);
+            bad |= (out & WALK_BAD) != 0;
+            st |= out & STOP_BITS;
+        }
+        __syncthreads();
+    }
+    if (act && !st && !carried) {
+        // MODE_FULL: usually nothing cuts any more; where something does, the
+        // pyramid walk clips by it (in its own order)
+        const int wr = window_walk<R, C>(slot, cp, lane);
+        if (MODE == MODE_CERTIFY && wr == WALK_STOP) st |= CS_UNCERTIFIED;
+        if (wr == WALK_OTHER || (MODE == MODE_FULL && wr == WALK_STOP)) {
             if (rec) {
                 if (lane == 0) P.ncert = 0;
-                if (lane < 27) P.supi[lane] = cert_sup(P.sup, lane);
                 __syncwarp();
             }
-            // near-first rings for cells clipped from a list; a warm-started cell of the
-            // FP64 re-clip already holds the FP32 pass's polytope, and the pyramid walk
-            // below clips every seed that cuts whatever the order
-            if (MODE == MODE_FULL && !(warm && cp.pass == 3))
-                done = ring_walk(P, cp, cc, b, zprev, lane, bad, st);
-            if (done) {
-                // MODE_FULL: usually nothing cuts any more; where something does, the
-                // pyramid walk clips by it (in its own order)
-                const int wr = window_walk(P, cp, cc, b, lane, bad, st);
-                if (MODE == MODE_CERTIFY) {
-                    if (wr == WALK_STOP) done = false;
-                } else if (wr == WALK_STOP) {
-                    st &= ~(uint32_t)CS_UNCERTIFIED;
-                }
-                if (wr == WALK_OTHER || (MODE == MODE_FULL && wr == WALK_STOP)) {
-                    if (rec) {
-                        if (lane == 0) P.ncert = 0;
-                        __syncwarp();
-                    }
-                    done = traverse<R, C, MODE>(P, cp, cc, b, lane, bad, st);
-                }
-            }
-            if (done && rec) {
-                __syncwarp();
-                ncert = P.ncert;
-                if (ncert >= 0) {
-                    cert_store(P, cp, b, i, lane);
-                    stored = true;
-                }
+            const uint32_t out = traverse<R, C, MODE>(slot, cp, lane);
+            bad |= (out & WALK_BAD) != 0;
+            st |= out & STOP_BITS;
+        }
+        if (!st && rec) {
+            __syncwarp();
+            ncert = P.ncert;
+            if (ncert >= 0) {
+                cert_store<R, C>(slot, cp, lane);
+                stored = true;
             }
         }
-        if (!done && MODE == MODE_CERTIFY && (st & CS_UNCERTIFIED)) {
-#ifdef SDOT_COUNTERS
-            __syncwarp();
-            if (lane < 8) atomicAdd(&cp.counters64[lane], (unsigned long long)P.wc[lane]);
-            __syncwarp();
-#endif
+        if (MODE == MODE_CERTIFY && (st & CS_UNCERTIFIED)) {
+            queued = true;
             if (lane == 0) {
                 const int32_t q = atomicAdd(cp.queue_cnt, 1);
                 cp.queue_out[q] = (int32_t)i;
                 cp.status[i] = (uint8_t)st;
                 cp.cert_n[i] = 0xff;
             }
-            return false;
         }
     }
 #ifdef SDOT_COUNTERS
-    __syncwarp();
-    if (lane < 8) atomicAdd(&cp.counters64[lane], (unsigned long long)P.wc[lane]);
-    __syncwarp();
+    if (act) {
+        __syncwarp();
+        if (lane < 8) atomicAdd(&cp.counters64[lane], (unsigned long long)P.wc[lane]);
+        __syncwarp();
+    }
 #endif
-    if (!st && cell_too_large(P, cc, psimax_glob, halfLmin, lane)) st |= CS_TOO_LARGE;
-    float cen[3];
-    bool have_cen = false;
-    if (!(st & (CS_EMPTY | CS_CAPACITY)))
-        have_cen = integrate(P, cp, cc.fr, i, lane, bad, st, cen);
-    // FP32 cells far from their frame origin (the first diagram of a context, or a
-    // large step of psi): clip again by the facets just found, in a frame at the
-    // centroid just found. The facets are the cell's complete neighbour set, so no
-    // walk is needed; the outputs are overwritten.
-    if (sizeof(R) == 4 && have_cen && !(st & (CS_EMPTY | CS_CAPACITY | CS_TOO_LARGE))) {
-        float dz2 = 0.f;
+    __syncthreads();
+    bool reframe = false;
+    if (act && !queued) {
+        if (!st && cell_too_large<R, C>(slot, psimax_glob, halfLmin, lane)) st |= CS_TOO_LARGE;
+        if (!(st & (CS_EMPTY | CS_CAPACITY))) {
+            const uint32_t r = integrate<R, C>(slot, cp, lane);
+            bad |= (r & CS_INCONSISTENT) != 0;
+            st |= r & (CS_CAPACITY | CS_CAP_FACE);
+            // FP32 cells far from their frame origin (the first diagram of a context, or a
+            // large step of psi): clip again by the facets just found, in a frame at the
+            // centroid just found. The facets are the cell's complete neighbour set, so no
+            // walk is needed; the outputs are overwritten.
+            if (sizeof(R) == 4 && (r & INT_VALID) &&
+                !(st & (CS_EMPTY | CS_CAPACITY | CS_TOO_LARGE))) {
+                float dz2 = 0.f;
 #pragma unroll
-        for (int a = 0; a < 3; a++) dz2 += (cen[a] - cc.fr.z[a]) * (cen[a] - cc.fr.z[a]);
-        if (dz2 > REFRAME_DIST * REFRAME_DIST) {
-            reframed = true;
-            __syncwarp();  // facets and counts written by integrate
-            const int nf = min(cp.fcnt[i], FCAP);
-            __syncwarp();
-            cc.fr = make_frame(cp, cen);
-            bad = false;
-            st = 0;
-            poly_init(P, cp, cc.fr.z, lane);
-            const int rc2 = clip_list(P, cp, cc, cp.fcol + i * FCAP, nf, lane, bad);
-            if (rc2 == CLIP_EMPTY) st |= CS_EMPTY;
-            if (rc2 == CLIP_CAP) st |= CS_CAPACITY | CS_CAP_POLY;
-            if (!st && cell_too_large(P, cc, psimax_glob, halfLmin, lane)) st |= CS_TOO_LARGE;
-            if (!(st & (CS_EMPTY | CS_CAPACITY))) integrate(P, cp, cc.fr, i, lane, bad, st, cen);
+                for (int a = 0; a < 3; a++)
+                    dz2 += (P.cen[a] - P.cc.fr.z[a]) * (P.cen[a] - P.cc.fr.z[a]);
+                reframe = dz2 > REFRAME_DIST * REFRAME_DIST;
+            }
         }
     }
+    if (sizeof(R) == 4 && __syncthreads_or(reframe)) {
+        if (reframe) {
+            const int nf = min(cp.fcnt[i], FCAP);
+            __syncwarp();
+            if (lane < 3) frame_axis(cp, P.cen[lane], lane, P.cc.fr);
+            __syncwarp();
+            st = 0;
+            poly_init<R, C>(slot, cp, lane);
+            const int rc = clip_list<R, C>(slot, cp, cp.fcol + i * FCAP, nf, lane);
+            bad = (rc & CLIP_BAD) != 0;
+            if ((rc & 3) == CLIP_EMPTY) st |= CS_EMPTY;
+            if ((rc & 3) == CLIP_CAP) st |= CS_CAPACITY | CS_CAP_POLY;
+        }
+        __syncthreads();
+        if (reframe) {
+            if (!st && cell_too_large<R, C>(slot, psimax_glob, halfLmin, lane)) st |= CS_TOO_LARGE;
+            if (!(st & (CS_EMPTY | CS_CAPACITY))) {
+                const uint32_t r = integrate<R, C>(slot, cp, lane);
+                bad |= (r & CS_INCONSISTENT) != 0;
+                st |= r & (CS_CAPACITY | CS_CAP_FACE);
+            }
+        }
+    }
+    if (!act || queued) return false;
     if (bad) st |= CS_INCONSISTENT;
     if (lane == 0) {
         if (st & (CS_EMPTY | CS_CAPACITY)) {
@@ -2032,7 +2073,7 @@ __device__ __forceinline__ bool process_cell(Poly<R, C>& P, const ClipParams& cp
         // the certificate stays valid only for a clean cell whose every plane other
         // than the box's is a facet (the planes of its next warm start); a first-pass
         // cell whose only failure is the FP32 check keeps it for its FP64 re-clip
-        const bool facets = !reframed && cp.fcnt[i] == P.np - 6;
+        const bool facets = !reframe && cp.fcnt[i] == P.np - 6;
         const bool keep1 = rec && facets && (carried || stored) &&
                            (st == 0 || (redo && st == CS_INCONSISTENT));
         const bool keep3 = use3 && facets && carried && st == 0;
@@ -2050,7 +2091,8 @@ namespace sdot {
 // centre of the vertices' bounding box, the faces found as in integrate. Every lane
 // gets the value; 0 when a face cycle is broken.
 template <typename R, class C>
-__device__ __noinline__ double poly_volume(Poly<R, C>& P, int lane) {
+__device__ __noinline__ double poly_volume(int slot, int lane) {
+    Poly<R, C>& P = poly_at<R, C>(slot);
     constexpr int FPL = (C::MP + 31) / 32;
     R o[3];
     {
@@ -2163,9 +2205,11 @@ __device__ __noinline__ double poly_volume(Poly<R, C>& P, int lane) {
     return ok ? vol6 / 6.0 : 0.0;
 }
 
-// P2 <- P1 (warp-uniform)
+// polytope slot2 <- slot1 (warp-uniform)
 template <typename R, class C>
-__device__ __noinline__ void poly_copy(Poly<R, C>& P2, const Poly<R, C>& P1, int lane) {
+__device__ __noinline__ void poly_copy(int slot2, int slot1, int lane) {
+    const Poly<R, C>& P1 = poly_at<R, C>(slot1);
+    Poly<R, C>& P2 = poly_at<R, C>(slot2);
     for (int q = lane; q < P1.np; q += 32) {
         P2.pl[q] = P1.pl[q];
         P2.plen[q] = P1.plen[q];

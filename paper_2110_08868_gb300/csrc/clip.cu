@@ -16,32 +16,40 @@
 
 namespace sdot {
 
-constexpr int WARPS_PER_BLOCK_CLIP = 4;
+// A block's warps go through the phases of a cell together (see process_cell). Larger
+// blocks keep the instruction cache better, smaller ones wait less for their slowest cell.
+// 1, 2, 4, 8 blocks per SM (32 to 4 warps each): first diagram 97^3, whose cells differ
+// most, 191, 148, 132, 138 ms; early Newton step 100^3 119, 111, 121, 146 ms; late step
+// 129^3 75, 60, 53, 55 ms.
+constexpr int CLIP_BLOCKS_PER_SM = 4;
 
-// resident blocks per SM a polytope size allows (shared memory), at most 8
+// Warps of a full clipping block: as many as shared memory holds polytopes for with
+// CLIP_BLOCKS_PER_SM blocks on an SM, and at most 32 warps an SM (64 registers a thread).
 template <typename R, class C>
-constexpr int clip_min_blocks() {
-    return (int)((227u * 1024u) / (WARPS_PER_BLOCK_CLIP * sizeof(Poly<R, C>))) < 8
-               ? (int)((227u * 1024u) / (WARPS_PER_BLOCK_CLIP * sizeof(Poly<R, C>)))
-               : 8;
+constexpr int clip_warps() {
+    return (int)((226u * 1024u / CLIP_BLOCKS_PER_SM - 1024u) / sizeof(Poly<R, C>)) <
+                   32 / CLIP_BLOCKS_PER_SM
+               ? (int)((226u * 1024u / CLIP_BLOCKS_PER_SM - 1024u) / sizeof(Poly<R, C>))
+               : 32 / CLIP_BLOCKS_PER_SM;
 }
 
 template <typename R, class C, int MODE>
-__global__ void __launch_bounds__(WARPS_PER_BLOCK_CLIP * 32, (clip_min_blocks<R, C>()))
+__global__ void __launch_bounds__(clip_warps<R, C>() * 32, CLIP_BLOCKS_PER_SM)
     clip_kernel(const __grid_constant__ ClipParams cp) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Poly<R, C>* polys = reinterpret_cast<Poly<R, C>*>(smem_raw);
-    const int lane = threadIdx.x & 31;
-    Poly<R, C>& P = polys[threadIdx.x >> 5];
+    __shared__ int64_t first;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const float psimax_glob = top_psimax(cp, lane);
     const float halfLmin = 0.5f * fminf(cp.Lt[0], fminf(cp.Lt[1], cp.Lt[2]));
     int carried = 0;  // cells certified by a carried certificate
     while (true) {
-        int64_t w = 0;
-        if (lane == 0) w = atomicAdd(cp.work_counter, 1);
-        w = __shfl_sync(FULLMASK, w, 0);
-        if (w >= cp.nwork) break;
-        carried += process_cell<R, C, MODE>(P, cp, w, psimax_glob, halfLmin, lane) ? 1 : 0;
+        __syncthreads();
+        if (threadIdx.x == 0) first = atomicAdd(cp.work_counter, nwarp);
+        __syncthreads();
+        const int64_t w = first + warp;
+        if (first >= cp.nwork) break;
+        carried += process_cell<R, C, MODE>(warp, cp, w < cp.nwork, w, psimax_glob, halfLmin, lane)
+                       ? 1
+                       : 0;
     }
     if (lane == 0 && carried) atomicAdd(cp.cert_carried, carried);
 }
@@ -57,18 +65,16 @@ struct ClipBatch {
 };
 
 template <typename R, class C, int MODE>
-__global__ void __launch_bounds__(WARPS_PER_BLOCK_CLIP * 32, (clip_min_blocks<R, C>()))
-    clip_batch_kernel(ClipBatch bt) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Poly<R, C>* polys = reinterpret_cast<Poly<R, C>*>(smem_raw);
-    const int lane = threadIdx.x & 31;
-    Poly<R, C>& P = polys[threadIdx.x >> 5];
+__global__ void __launch_bounds__(clip_warps<R, C>() * 32, CLIP_BLOCKS_PER_SM) clip_batch_kernel(ClipBatch bt) {
+    __shared__ long long first;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const long long total = bt.start[bt.njobs];
     while (true) {
-        long long w = 0;
-        if (lane == 0) w = (long long)atomicAdd(bt.counter, 1ull);
-        w = __shfl_sync(FULLMASK, w, 0);
-        if (w >= total) break;
+        __syncthreads();
+        if (threadIdx.x == 0) first = (long long)atomicAdd(bt.counter, (unsigned long long)nwarp);
+        __syncthreads();
+        const long long w = first + warp;
+        if (first >= total) break;
         // the last job j with start[j] <= w (jobs without items are skipped)
         int lo = 0, hi = bt.njobs - 1;
         while (lo < hi) {
@@ -79,8 +85,8 @@ __global__ void __launch_bounds__(WARPS_PER_BLOCK_CLIP * 32, (clip_min_blocks<R,
         const ClipParams& cp = bt.jobs[lo];
         const float psimax_glob = top_psimax(cp, lane);
         const float halfLmin = 0.5f * fminf(cp.Lt[0], fminf(cp.Lt[1], cp.Lt[2]));
-        process_cell<R, C, MODE>(P, cp, (int64_t)(w - bt.start[lo]), psimax_glob, halfLmin,
-                                 lane);
+        process_cell<R, C, MODE>(warp, cp, w < total, (int64_t)(w - bt.start[lo]), psimax_glob,
+                                 halfLmin, lane);
     }
 }
 
@@ -268,72 +274,37 @@ __global__ void cell_reduce_final(const double* __restrict__ part, int nb, doubl
     out[5] = (double)fl;
 }
 
-// Setup of a persistent clipping kernel, once per instantiation: blocks per SM from the
-// occupancy at the largest shared-memory carveout, then the smallest carveout that still
-// holds that many blocks, so the rest of the SM's memory stays L1 (which caches the
-// lanes' local memory). The occupancy is checked again at that carveout and the largest
-// one restored if it dropped.
-template <typename K>
-static cudaError_t clip_setup(K kernel, size_t smem, int* blocks) {
-    const int threads = WARPS_PER_BLOCK_CLIP * 32;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    int per_sm = 0;
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    int dev = 0, smem_sm = 0, resv = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) ==
-            cudaSuccess &&
-        cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev) ==
-            cudaSuccess &&
-        smem_sm > 0) {
-        // shared memory is allocated per block in 128-byte units, plus the reserved part;
-        // the percentage is rounded down and the driver rounds it up to a supported size
-        const size_t per_block = (smem + (size_t)resv + 127) / 128 * 128;
-        const int pct = (int)((size_t)per_sm * per_block * 100 / (size_t)smem_sm);
-        if (pct < 100 &&
-            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct) ==
-                cudaSuccess) {
-            int again = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&again, kernel, threads, smem) !=
-                    cudaSuccess ||
-                again < per_sm)
-                cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        }
-        cudaGetLastError();
-    }
-    *blocks = per_sm * num_sms();
-    return cudaSuccess;
+// Warps of a clipping block and blocks for nwork cells: full blocks where there are cells
+// for one on every SM, smaller ones (the cells spread over all SMs) below that.
+struct ClipGrid {
+    int warps, blocks;
+};
+template <typename R, class C>
+static ClipGrid clip_grid(int64_t nwork) {
+    const int sms = num_sms();
+    const int64_t per_block = (nwork + sms - 1) / sms;
+    ClipGrid g;
+    g.warps = per_block < clip_warps<R, C>() ? (int)per_block : clip_warps<R, C>();
+    const int64_t need = (nwork + g.warps - 1) / g.warps;
+    const int most = sms * CLIP_BLOCKS_PER_SM;
+    g.blocks = (int)(need < most ? need : most);
+    return g;
 }
 
 template <typename R, class C, int MODE>
 static int launch_clip(const ClipParams& cp, cudaStream_t s) {
-    const size_t smem = sizeof(Poly<R, C>) * WARPS_PER_BLOCK_CLIP;
-    // kernel attributes and the persistent grid size, set once per instantiation
-    // (thread-safe: contexts of different host threads launch concurrently)
-    struct Setup {
-        int blocks;
-        cudaError_t err;
-    };
-    static const Setup setup = [smem] {
-        Setup u{0, cudaSuccess};
-        u.err = clip_setup(clip_kernel<R, C, MODE>, smem, &u.blocks);
-        return u;
-    }();
-    if (setup.err != cudaSuccess) {
-        set_error(std::string("clip kernel setup: ") + cudaGetErrorString(setup.err));
+    // the shared-memory limit, raised once per instantiation (thread-safe: contexts of
+    // different host threads launch concurrently)
+    static const cudaError_t err = cudaFuncSetAttribute(
+        clip_kernel<R, C, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)(sizeof(Poly<R, C>) * clip_warps<R, C>()));
+    if (err != cudaSuccess) {
+        set_error(std::string("clip kernel setup: ") + cudaGetErrorString(err));
         return SDOT_ERR_CUDA;
     }
-    const int blocks = setup.blocks;
-    int64_t need = (cp.nwork + WARPS_PER_BLOCK_CLIP - 1) / WARPS_PER_BLOCK_CLIP;
-    int nb = (int)(need < blocks ? need : blocks);
-    if (nb < 1) return SDOT_OK;
-    clip_kernel<R, C, MODE><<<nb, WARPS_PER_BLOCK_CLIP * 32, smem, s>>>(cp);
+    if (cp.nwork < 1) return SDOT_OK;
+    const ClipGrid g = clip_grid<R, C>(cp.nwork);
+    clip_kernel<R, C, MODE><<<g.blocks, g.warps * 32, sizeof(Poly<R, C>) * g.warps, s>>>(cp);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     return SDOT_OK;
@@ -507,24 +478,16 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
 // ---------------------------------------------------------------------------
 template <typename R, class C, int MODE>
 static int launch_clip_batch(const ClipBatch& bt, int64_t total, cudaStream_t s) {
-    const size_t smem = sizeof(Poly<R, C>) * WARPS_PER_BLOCK_CLIP;
-    struct Setup {
-        int blocks;
-        cudaError_t err;
-    };
-    static const Setup setup = [smem] {
-        Setup u{0, cudaSuccess};
-        u.err = clip_setup(clip_batch_kernel<R, C, MODE>, smem, &u.blocks);
-        return u;
-    }();
-    if (setup.err != cudaSuccess) {
-        set_error(std::string("clip batch kernel setup: ") + cudaGetErrorString(setup.err));
+    static const cudaError_t err = cudaFuncSetAttribute(
+        clip_batch_kernel<R, C, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)(sizeof(Poly<R, C>) * clip_warps<R, C>()));
+    if (err != cudaSuccess) {
+        set_error(std::string("clip batch kernel setup: ") + cudaGetErrorString(err));
         return SDOT_ERR_CUDA;
     }
-    const int64_t need = (total + WARPS_PER_BLOCK_CLIP - 1) / WARPS_PER_BLOCK_CLIP;
-    const int nb = (int)(need < setup.blocks ? need : setup.blocks);
-    if (nb < 1) return SDOT_OK;
-    clip_batch_kernel<R, C, MODE><<<nb, WARPS_PER_BLOCK_CLIP * 32, smem, s>>>(bt);
+    if (total < 1) return SDOT_OK;
+    const ClipGrid g = clip_grid<R, C>(total);
+    clip_batch_kernel<R, C, MODE><<<g.blocks, g.warps * 32, sizeof(Poly<R, C>) * g.warps, s>>>(bt);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     return SDOT_OK;

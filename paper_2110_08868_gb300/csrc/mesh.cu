@@ -66,29 +66,22 @@ constexpr int MESH_WARPS = 2;
 
 __global__ void __launch_bounds__(MESH_WARPS * 32)
     mesh_kernel(const __grid_constant__ ClipParams cp, const __grid_constant__ MeshParams mp) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     using PolyT = Poly<double, MeshCap>;
-    PolyT* polys = reinterpret_cast<PolyT*>(smem_raw);
     const int lane = threadIdx.x & 31;
-    PolyT& P = polys[2 * (threadIdx.x >> 5)];
-    PolyT& Q = polys[2 * (threadIdx.x >> 5) + 1];
+    const int ps = 2 * (threadIdx.x >> 5), qs = ps + 1;
+    PolyT& P = poly_at<double, MeshCap>(ps);
     const int M = mp.M;
     while (true) {
         int64_t i = 0;
         if (lane == 0) i = atomicAdd(mp.work, 1);
         i = __shfl_sync(FULLMASK, i, 0);
         if (i >= cp.N) break;
-        CellCtx cc;
-        cc.i = i;
-        cc.yi = cp.pos[i];
-        cc.psii = cp.psi[i];
-        cc.si = load_seed(cp, i);
-        cc.fr = seed_frame();
-        bool bad = false;
-        poly_init(P, cp, cc.fr.z, lane);
+        load_cell<double, MeshCap>(ps, cp, i, lane);
+        const CellCtx& cc = P.cc;
+        poly_init<double, MeshCap>(ps, cp, lane);
         const int nf = min(cp.fcnt[i], FCAP);
-        const int rc = clip_list(P, cp, cc, cp.fcol + i * FCAP, nf, lane, bad);
-        if (rc == CLIP_EMPTY || rc == CLIP_CAP || bad) {
+        const int rc = clip_list<double, MeshCap>(ps, cp, cp.fcol + i * FCAP, nf, lane);
+        if (rc != CLIP_NONE) {
             if (lane == 0) atomicAdd(mp.flags, 1);
             continue;
         }
@@ -150,7 +143,7 @@ __global__ void __launch_bounds__(MESH_WARPS * 32)
         }
         if (mp.pass != 0 || !mp.mass_fx) continue;
         // --- deposit: the cell against every pulled-back voxel it meets --------------
-        const double volP = poly_volume(P, lane);
+        const double volP = poly_volume<double, MeshCap>(ps, lane);
         if (!(volP > 0.0)) {
             if (lane == 0) atomicAdd(mp.flags, 1);
             continue;
@@ -165,7 +158,7 @@ __global__ void __launch_bounds__(MESH_WARPS * 32)
             for (long long vy = v0[1]; vy <= v1[1]; vy++)
                 for (long long vx = v0[0]; vx <= v1[0]; vx++) {
                     const long long vv[3] = {vx, vy, vz};
-                    poly_copy(Q, P, lane);
+                    poly_copy<double, MeshCap>(qs, ps, lane);
                     bool empty = false, qbad = false;
                     for (int a = 0; a < 3 && !empty; a++) {
                         // voxel [v h, (v + 1) h] pulled back: p in [(v h - y)/s, ((v+1) h - y)/s]
@@ -176,7 +169,8 @@ __global__ void __launch_bounds__(MESH_WARPS * 32)
                         pn.y = a == 1 ? 1.0 : 0.0;
                         pn.z = a == 2 ? 1.0 : 0.0;
                         pn.w = bhi;
-                        int r = poly_clip(Q, pn, 1.0, -2, lane, qbad);
+                        int r = poly_clip<double, MeshCap>(qs, pn, 1.0, -2, lane);
+                        if (r & CLIP_BAD) qbad = true;
                         if (r == CLIP_EMPTY) empty = true;
                         if (r == CLIP_CAP) {
                             qbad = true;
@@ -187,7 +181,8 @@ __global__ void __launch_bounds__(MESH_WARPS * 32)
                         pn.y = -pn.y;
                         pn.z = -pn.z;
                         pn.w = -blo;
-                        r = poly_clip(Q, pn, 1.0, -2, lane, qbad);
+                        r = poly_clip<double, MeshCap>(qs, pn, 1.0, -2, lane);
+                        if (r & CLIP_BAD) qbad = true;
                         if (r == CLIP_EMPTY) empty = true;
                         if (r == CLIP_CAP) {
                             qbad = true;
@@ -196,7 +191,7 @@ __global__ void __launch_bounds__(MESH_WARPS * 32)
                     }
                     if (qbad && lane == 0) atomicAdd(mp.flags, 1);
                     if (empty) continue;
-                    const double vq = poly_volume(Q, lane);
+                    const double vq = poly_volume<double, MeshCap>(qs, lane);
                     if (!(vq > 0.0)) continue;
                     if (lane == 0) {
                         const double c = nui * (vq / volP);
