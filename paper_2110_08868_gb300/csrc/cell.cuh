@@ -194,6 +194,7 @@ struct ClipParams {
     int32_t* work_counter;
     const int32_t* worklist;  // null: cells 0..nwork-1
     int64_t nwork;
+    const int32_t* nwork_dev;        // not null: the work items, counted on the device
     unsigned long long* counters64;  // diagnostic work counters (8)
     const float* pslo;               // low part of psi/a^2
     const uint4* ioff;               // grid-cell offsets, 32-bit fixed point
@@ -304,11 +305,11 @@ __device__ __noinline__ void poly_init(int slot, const ClipParams& cp, int lane)
     __syncwarp();
 }
 
-// The vertex of planes (a, b, c) of t; well: the triple is well conditioned,
+// The vertex of three planes; well: the triple is well conditioned,
 // det(n_a, n_b, n_c) > dtol |n_a| |n_b| |n_c|.
-template <typename R, class C>
-__device__ __forceinline__ V3<R> vertex_of(const Poly<R, C>& P, uint32_t t, R dtol, bool& well) {
-    const V4<R> A = P.pl[t & 0xff], B = P.pl[(t >> 8) & 0xff], Cc = P.pl[(t >> 16) & 0xff];
+template <typename R>
+__device__ __forceinline__ V3<R> vertex_of3(const V4<R>& A, const V4<R>& B, const V4<R>& Cc, R la,
+                                            R lb, R lc, R dtol, bool& well) {
     // n_b x n_c, n_c x n_a, n_a x n_b
     R bcx = B.y * Cc.z - B.z * Cc.y, bcy = B.z * Cc.x - B.x * Cc.z, bcz = B.x * Cc.y - B.y * Cc.x;
     R cax = Cc.y * A.z - Cc.z * A.y, cay = Cc.z * A.x - Cc.x * A.z, caz = Cc.x * A.y - Cc.y * A.x;
@@ -319,9 +320,15 @@ __device__ __forceinline__ V3<R> vertex_of(const Poly<R, C>& P, uint32_t t, R dt
     v.x = (A.w * bcx + B.w * cax + Cc.w * abx) * inv;
     v.y = (A.w * bcy + B.w * cay + Cc.w * aby) * inv;
     v.z = (A.w * bcz + B.w * caz + Cc.w * abz) * inv;
-    R la = P.plen[t & 0xff], lb = P.plen[(t >> 8) & 0xff], lc = P.plen[(t >> 16) & 0xff];
     well = det > dtol * (la * lb * lc);
     return v;
+}
+// the vertex of planes (a, b, c) of t
+template <typename R, class C>
+__device__ __forceinline__ V3<R> vertex_of(const Poly<R, C>& P, uint32_t t, R dtol, bool& well) {
+    const V4<R> A = P.pl[t & 0xff], B = P.pl[(t >> 8) & 0xff], Cc = P.pl[(t >> 16) & 0xff];
+    const R la = P.plen[t & 0xff], lb = P.plen[(t >> 8) & 0xff], lc = P.plen[(t >> 16) & 0xff];
+    return vertex_of3(A, B, Cc, la, lb, lc, dtol, well);
 }
 
 // drop planes no vertex references any more; returns the number of planes left
@@ -1349,6 +1356,35 @@ __device__ __noinline__ int window_walk(int slot, const ClipParams& cp, int lane
     return WALK_DONE;
 }
 
+// normals less than 0.03 rad from parallel (the angle of the FP32 consistency check)
+template <typename R>
+__device__ __forceinline__ bool nearly_parallel(const V4<R>& A, const V4<R>& B) {
+    constexpr float SIN2_MIN = 0.03f * 0.03f;
+    const float la2 = A.x * A.x + A.y * A.y + A.z * A.z;
+    const float lb2 = B.x * B.x + B.y * B.y + B.z * B.z;
+    const float x = A.y * B.z - A.z * B.y, y = A.z * B.x - A.x * B.z, z = A.x * B.y - A.y * B.x;
+    return x * x + y * y + z * z < SIN2_MIN * la2 * lb2;
+}
+
+// One triangle (v0, vp, vc) of a face's fan, vertices relative to o: its area vector, and
+// the volume (times 6) and first moment (times 24) of its tetrahedron with o.
+template <typename R>
+__device__ __forceinline__ void fan_triangle(const V3<R>& v0, const V3<R>& vp, const V3<R>& vc, R& Sx,
+                                             R& Sy, R& Sz, R& fv6, R& fmx, R& fmy, R& fmz) {
+    const R ax = vp.x - v0.x, ay = vp.y - v0.y, az = vp.z - v0.z;
+    const R bx = vc.x - v0.x, by = vc.y - v0.y, bz = vc.z - v0.z;
+    const R cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
+    Sx += cx;
+    Sy += cy;
+    Sz += cz;
+    // 6 |tet(o, v0, vp, vc)| = det(v0, vp, vc) with vertices relative to o
+    const R d6 = v0.x * cx + v0.y * cy + v0.z * cz;
+    fv6 += d6;
+    fmx += d6 * (v0.x + vp.x + vc.x);
+    fmy += d6 * (v0.y + vp.y + vc.y);
+    fmz += d6 * (v0.z + vp.z + vc.z);
+}
+
 // Integrate the polytope and write the outputs of its cell; P.cen receives the centroid
 // relative to the seed (units of a). Returns status bits: CS_CAPACITY, CS_INCONSISTENT for a
 // failed check, INT_VALID when the centroid is valid (positive finite volume).
@@ -1370,27 +1406,15 @@ __device__ __noinline__ uint32_t integrate(int slot, const ClipParams& cp, int l
     // is off by about (plane rounding) / angle, far above the cell's own rounding; such a
     // cell fails the check and is clipped again in FP64. Box planes take no part.
     if (sizeof(R) == 4) {
-        constexpr float SIN2_MIN = 0.03f * 0.03f;  // ANGLE_MIN = 0.03 rad
         bool ill = false;
 #pragma unroll 1
         for (int s2 = lane; s2 < P.nt; s2 += 32) {
             const uint32_t t = P.tri[s2];
             const uint32_t ia = t & 0xff, ib = (t >> 8) & 0xff, ic = (t >> 16) & 0xff;
             const V4<R> A = P.pl[ia], Bq = P.pl[ib], Cq = P.pl[ic];
-            const float la2 = A.x * A.x + A.y * A.y + A.z * A.z;
-            const float lb2 = Bq.x * Bq.x + Bq.y * Bq.y + Bq.z * Bq.z;
-            const float lc2 = Cq.x * Cq.x + Cq.y * Cq.y + Cq.z * Cq.z;
-            const float bcx = Bq.y * Cq.z - Bq.z * Cq.y, bcy = Bq.z * Cq.x - Bq.x * Cq.z,
-                        bcz = Bq.x * Cq.y - Bq.y * Cq.x;
-            const float cax = Cq.y * A.z - Cq.z * A.y, cay = Cq.z * A.x - Cq.x * A.z,
-                        caz = Cq.x * A.y - Cq.y * A.x;
-            const float abx = A.y * Bq.z - A.z * Bq.y, aby = A.z * Bq.x - A.x * Bq.z,
-                        abz = A.x * Bq.y - A.y * Bq.x;
-            if (ia >= 6 && ib >= 6 && abx * abx + aby * aby + abz * abz < SIN2_MIN * la2 * lb2)
-                ill = true;
-            if (ib >= 6 && ic >= 6 && bcx * bcx + bcy * bcy + bcz * bcz < SIN2_MIN * lb2 * lc2)
-                ill = true;
-            if (ic >= 6 && ia >= 6 && cax * cax + cay * cay + caz * caz < SIN2_MIN * lc2 * la2)
+            if ((ia >= 6 && ib >= 6 && nearly_parallel(A, Bq)) ||
+                (ib >= 6 && ic >= 6 && nearly_parallel(Bq, Cq)) ||
+                (ic >= 6 && ia >= 6 && nearly_parallel(Cq, A)))
                 ill = true;
         }
         if (__any_sync(FULLMASK, ill)) bad = true;
@@ -1506,21 +1530,7 @@ __device__ __noinline__ uint32_t integrate(int slot, const ClipParams& cp, int l
             vc.x -= o[0];
             vc.y -= o[1];
             vc.z -= o[2];
-            if (step >= 2) {
-                // fan triangle (v0, vp, vc) and tetrahedron (o, v0, vp, vc)
-                const R ax = vp.x - v0.x, ay = vp.y - v0.y, az = vp.z - v0.z;
-                const R bx = vc.x - v0.x, by = vc.y - v0.y, bz = vc.z - v0.z;
-                const R cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-                Sx += cx;
-                Sy += cy;
-                Sz += cz;
-                // 6 |tet(o, v0, vp, vc)| = det(v0, vp, vc) with vertices relative to o
-                const R d6 = v0.x * cx + v0.y * cy + v0.z * cz;
-                fv6 += d6;
-                fmx += d6 * (v0.x + vp.x + vc.x);
-                fmy += d6 * (v0.y + vp.y + vc.y);
-                fmz += d6 * (v0.z + vp.z + vc.z);
-            }
+            if (step >= 2) fan_triangle(v0, vp, vc, Sx, Sy, Sz, fv6, fmx, fmy, fmz);
             vp = vc;
         }
         if (ok && ((ecur >> 8) & 0xff) != x0) ok = false;

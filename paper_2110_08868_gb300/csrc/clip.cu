@@ -16,6 +16,9 @@
 
 namespace sdot {
 
+// carry.cu: the cells a carried certificate certifies; the others go to queue (count cnt)
+int launch_carry(const ClipParams& cp, int32_t* queue, int32_t* cnt, int32_t* work, cudaStream_t s);
+
 // A block's warps go through the phases of a cell together (see process_cell). Larger
 // blocks keep the instruction cache better, smaller ones wait less for their slowest cell.
 // 1, 2, 4, 8 blocks per SM (32 to 4 warps each): first diagram 97^3, whose cells differ
@@ -40,14 +43,15 @@ __global__ void __launch_bounds__(clip_warps<R, C>() * 32, CLIP_BLOCKS_PER_SM)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const float psimax_glob = top_psimax(cp, lane);
     const float halfLmin = 0.5f * fminf(cp.Lt[0], fminf(cp.Lt[1], cp.Lt[2]));
+    const int64_t nwork = cp.nwork_dev ? *cp.nwork_dev : cp.nwork;
     int carried = 0;  // cells certified by a carried certificate
     while (true) {
         __syncthreads();
         if (threadIdx.x == 0) first = atomicAdd(cp.work_counter, nwarp);
         __syncthreads();
         const int64_t w = first + warp;
-        if (first >= cp.nwork) break;
-        carried += process_cell<R, C, MODE>(warp, cp, w < cp.nwork, w, psimax_glob, halfLmin, lane)
+        if (first >= nwork) break;
+        carried += process_cell<R, C, MODE>(warp, cp, w < nwork, w, psimax_glob, halfLmin, lane)
                        ? 1
                        : 0;
     }
@@ -365,6 +369,7 @@ static ClipParams make_clip_params(DeviceState& d, const double* psi) {
     cp.work_counter = nullptr;
     cp.worklist = nullptr;
     cp.nwork = d.N;
+    cp.nwork_dev = nullptr;
     cp.pass = 1;
     return cp;
 }
@@ -373,28 +378,37 @@ static ClipParams make_clip_params(DeviceState& d, const double* psi) {
 // FP64 (mesh.cu)
 ClipParams mesh_clip_params(DeviceState& d) { return make_clip_params(d, d.psi); }
 
+// The carried pass runs for FP32 cells that may hold a certificate. Its queue lies in
+// rowcnt, which the CSR assembly rewrites.
+static bool carries(const DeviceState& d, int precision) {
+    return precision != SDOT_PREC_FP64 && d.carry && d.facets_valid;
+}
+
 int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult* res,
                    cudaStream_t s) {
     NvtxRange nv("laguerre_cells");
     int rc = build_pyramid(d, psi, s);
     if (rc) return rc;
     ClipParams cp = make_clip_params(d, psi);
-    SDOT_CUDA_TRY(cudaMemsetAsync(d.counters, 0, 8 * sizeof(int32_t), s));
-    SDOT_CUDA_TRY(cudaMemsetAsync(d.counters + 29, 0, sizeof(int32_t), s));
+    SDOT_CUDA_TRY(cudaMemsetAsync(d.counters, 0, 30 * sizeof(int32_t), s));
 
     cudaEvent_t e0, e1, ep1, ep2;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventCreate(&ep1);
     cudaEventCreate(&ep2);
-    cp.counters64 = (unsigned long long*)(d.counters + 8);
-    SDOT_CUDA_TRY(cudaMemsetAsync(d.counters + 8, 0, 64, s));
     cudaEventRecord(e0, s);
-    // pass 1: every cell, kNN planes + security test
+    // pass 1: every cell, first candidates + security test; before it, where certificates
+    // may hold, the cells they carry
     cp.work_counter = d.counters + 2;
     cp.worklist = nullptr;
     cp.nwork = d.N;
     cp.pass = 1;
+    if (carries(d, precision)) {
+        cp.worklist = d.rowcnt;
+        cp.nwork_dev = d.counters + 7;
+        if ((rc = launch_carry(cp, d.rowcnt, d.counters + 7, d.counters + 25, s))) return rc;
+    }
     rc = precision == SDOT_PREC_FP64 ? launch_clip<double, CapS, MODE_CERTIFY>(cp, s)
                                      : launch_clip<float, CapS, MODE_CERTIFY>(cp, s);
     if (rc) return rc;
@@ -408,6 +422,7 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
         cp.work_counter = d.counters + 4;
         cp.worklist = d.queue;
         cp.nwork = requeued;
+        cp.nwork_dev = nullptr;
         cp.pass = 2;
         rc = precision == SDOT_PREC_FP64 ? launch_clip<double, CapS, MODE_FULL>(cp, s)
                                          : launch_clip<float, CapS, MODE_FULL>(cp, s);
@@ -425,6 +440,7 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
         cp.work_counter = d.counters + 5;
         cp.worklist = d.queue64;
         cp.nwork = reclipped;
+        cp.nwork_dev = nullptr;
         if (precision != SDOT_PREC_FP64) {
             if ((rc = launch_clip<double, CapS, MODE_FULL>(cp, s))) return rc;
             SDOT_CUDA_TRY(cudaMemcpyAsync(cnt, d.counters, 8, cudaMemcpyDeviceToHost, s));
@@ -602,8 +618,7 @@ int evaluate_cells_batch(DeviceState* const* ds, const double* const* psis, cons
         DeviceState& d = *ds[j];
         if ((rc = build_pyramid(d, psis[j], s))) return rc;
         cps[j] = make_clip_params(d, psis[j]);
-        SDOT_CUDA_TRY(cudaMemsetAsync(d.counters, 0, 8 * sizeof(int32_t), s));
-        SDOT_CUDA_TRY(cudaMemsetAsync(d.counters + 8, 0, 64, s));
+        SDOT_CUDA_TRY(cudaMemsetAsync(d.counters, 0, 30 * sizeof(int32_t), s));
         is64[j] = precs[j] == SDOT_PREC_FP64;
         is32[j] = !is64[j];
     }
@@ -619,11 +634,36 @@ int evaluate_cells_batch(DeviceState* const* ds, const double* const* psis, cons
         cudaEventDestroy(ep2);
     };
     cudaEventRecord(e0, s);
-    // pass 1: every cell of every job
+    // pass 1: every cell of every job, less those a certificate carries (each job's carried
+    // pass comes first and leaves the rest in its queue)
+    bool carry = false;
     for (int j = 0; j < n; j++) {
+        DeviceState& d = *ds[j];
         cps[j].worklist = nullptr;
         cps[j].pass = 1;
-        nwork[j] = ds[j]->N;
+        nwork[j] = d.N;
+        if (!carries(d, precs[j])) continue;
+        cps[j].worklist = d.rowcnt;
+        rc = launch_carry(cps[j], d.rowcnt, d.counters + 7, d.counters + 25, s);
+        if (!rc && cudaMemcpyAsync(sc->cnt_host + 2 * j, d.counters + 7, sizeof(int32_t),
+                                   cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+            set_error("evaluate_cells_batch: reading a queue's count failed");
+            rc = SDOT_ERR_CUDA;
+        }
+        if (rc) {
+            cleanup();
+            return rc;
+        }
+        carry = true;
+    }
+    if (carry) {
+        if (cudaStreamSynchronize(s) != cudaSuccess) {
+            cleanup();
+            set_error("evaluate_cells_batch: the carried pass failed");
+            return SDOT_ERR_CUDA;
+        }
+        for (int j = 0; j < n; j++)
+            if (cps[j].worklist) nwork[j] = sc->cnt_host[2 * j];
     }
     if ((rc = launch_table<float, CapS, MODE_CERTIFY>(cps, nwork, is32, 0, sc, s)) ||
         (rc = launch_table<double, CapS, MODE_CERTIFY>(cps, nwork, is64, 1, sc, s))) {
