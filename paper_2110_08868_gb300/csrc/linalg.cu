@@ -48,6 +48,30 @@ __device__ __forceinline__ double sym_value(const int32_t* __restrict__ fcnt,
     return seen ? 0.5 * (cij + cji) : 0.0;
 }
 
+// Which of row j's facets are with cell i: bit u of the result. A row is 64 entries
+// (FCAP) of 4 bytes whatever its count, so its first 16 are asked for together with the
+// count: one round of loads for most rows (15.5 facets in the mean), where a loop over the
+// entries waited for the count and then took one load each.
+__device__ __forceinline__ uint64_t reports_of(const int32_t* __restrict__ fcnt,
+                                               const int32_t* __restrict__ fcol, int32_t j,
+                                               int32_t i) {
+    const int4* row = reinterpret_cast<const int4*>(fcol + (int64_t)j * FCAP);
+    const int nj = fcnt[j];
+    uint64_t m = 0;
+    auto group = [&](int4 q, int u) {
+        const uint32_t b = (q.x == i ? 1u : 0u) | (q.y == i ? 2u : 0u) | (q.z == i ? 4u : 0u) |
+                           (q.w == i ? 8u : 0u);
+        m |= (uint64_t)b << u;
+    };
+    const int4 q0 = row[0], q1 = row[1], q2 = row[2], q3 = row[3];
+    group(q0, 0);
+    group(q1, 4);
+    group(q2, 8);
+    group(q3, 12);
+    for (int u = 16; u < nj; u += 4) group(row[u >> 2], u);
+    return nj >= 64 ? m : m & ((1ull << nj) - 1ull);
+}
+
 // Row i's facets, one per lane (rows of at most 32 facets): the symmetrised
 // coefficient of each first occurrence of a column (sym_value's value, with the same
 // sums in the same order, so L stays exactly symmetric) and whether it enters L.
@@ -79,14 +103,11 @@ __device__ __forceinline__ RowSym row_sym_warp(const int32_t* __restrict__ fcnt,
     }
     double cji = 0.0;
     bool seen = false;
-    if (first) {
-        const int nj = fcnt[r.j];
-        for (int u = 0; u < nj; u++)
-            if (fcol[(int64_t)r.j * FCAP + u] == (int32_t)i) {
-                cji += fval[(int64_t)r.j * FCAP + u];
-                seen = true;
-            }
-    }
+    if (first)
+        for (uint64_t m = reports_of(fcnt, fcol, r.j, (int32_t)i); m; m &= m - 1) {
+            cji += fval[(int64_t)r.j * FCAP + __ffsll((long long)m) - 1];
+            seen = true;
+        }
     r.v = (first && seen) ? 0.5 * (cij + cji) : 0.0;
     r.keep = r.v > 0.0;
     return r;
@@ -153,10 +174,8 @@ __global__ void csr_fill_kernel(const int32_t* __restrict__ fcnt, const int32_t*
     const RowSym r = row_sym_warp(fcnt, fcol, fval, i, n, lane);
     const uint32_t km = __ballot_sync(FULLMASK, r.keep);
     int rank = 0;
-    for (int src = 0; src < 32; src++) {
-        const int32_t js = __shfl_sync(FULLMASK, r.j, src);
-        if (((km >> src) & 1u) && js < r.j) rank++;
-    }
+    for (uint32_t m = km; m; m &= m - 1)
+        if (__shfl_sync(FULLMASK, r.j, __ffs(m) - 1) < r.j) rank++;
     if (r.keep) {
         col[p0 + 1 + rank] = r.j;
         val[p0 + 1 + rank] = -r.v;
@@ -243,10 +262,8 @@ __global__ void csr_user_fill(const int64_t* __restrict__ row_ptr, const int32_t
     const int32_t j = act ? perm[col[b + 1 + lane]] : 0;
     const double v = act ? val[b + 1 + lane] : 0.0;
     int rank = 0;
-    for (int src = 0; src < 32; src++) {
-        const int32_t js = __shfl_sync(FULLMASK, j, src);
-        if (src < m && js < j) rank++;
-    }
+    for (int src = 0; src < m; src++)
+        if (__shfl_sync(FULLMASK, j, src) < j) rank++;
     if (act) {
         col_u[o + 1 + rank] = j;
         val_u[o + 1 + rank] = v;
@@ -287,75 +304,127 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return t;  // valid in thread 0
 }
 
-// Off-diagonal entries kept per row (symmetrised facets of positive weight); one warp
-// per slice of 32 rows, whose width (longest row) it records, and the total count.
-__global__ void sell_count_kernel(const int32_t* __restrict__ fcnt, const int32_t* __restrict__ fcol,
-                                  const double* __restrict__ fval, int64_t N, int64_t nslice,
-                                  int32_t* __restrict__ width, unsigned long long* __restrict__ nnz) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    unsigned long long tot = 0;
-    for (int64_t sl = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < nslice;
-         sl += nw) {
-        const int64_t i = sl * 32 + lane;
+// Entries row i keeps (symmetrised facets of positive weight), by the whole warp.
+__device__ __forceinline__ int row_kept(const int32_t* __restrict__ fcnt,
+                                        const int32_t* __restrict__ fcol,
+                                        const double* __restrict__ fval, int64_t i, int lane) {
+    const int n = fcnt[i];
+    if (n > 32) {  // rare: the row in lane 0, serially
         int kept = 0;
-        if (i < N) {
-            const int n = fcnt[i];
+        if (lane == 0)
             for (int t = 0; t < n; t++)
                 if (sym_value(fcnt, fcol, fval, i, t) > 0.0) kept++;
-        }
-        const int w = __reduce_max_sync(FULLMASK, kept);
-        if (lane == 0) width[sl] = w;
-        tot += (unsigned long long)__reduce_add_sync(FULLMASK, (unsigned)kept);
+        return __shfl_sync(FULLMASK, kept, 0);
     }
-    if (lane == 0 && tot) atomicAdd(nnz, tot);
+    return __popc(__ballot_sync(FULLMASK, row_sym_warp(fcnt, fcol, fval, i, n, lane).keep));
+}
+
+// One block per slice of 32 rows, one warp per row (four rows each): a row's facets are its
+// lanes, so the searches in the neighbours' rows run side by side (with a thread per row
+// they ran one after the other, and a 16^3 box had 128 warps at work). Records the slice's
+// width (its longest row) and the total count.
+constexpr int SELL_ROWS = 32 / (CG_THREADS / 32);  // rows a warp takes
+
+__global__ void __launch_bounds__(CG_THREADS)
+    sell_count_kernel(const int32_t* __restrict__ fcnt, const int32_t* __restrict__ fcol,
+                      const double* __restrict__ fval, int64_t N, int32_t* __restrict__ width,
+                      unsigned long long* __restrict__ nnz) {
+    __shared__ int most, sum;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) most = sum = 0;
+    __syncthreads();
+    int w = 0, tot = 0;
+    for (int q = 0; q < SELL_ROWS; q++) {
+        const int64_t i = (int64_t)blockIdx.x * 32 + warp * SELL_ROWS + q;
+        if (i >= N) break;
+        const int kept = row_kept(fcnt, fcol, fval, i, lane);
+        w = max(w, kept);
+        tot += kept;
+    }
+    if (lane == 0) {
+        atomicMax(&most, w);
+        atomicAdd(&sum, tot);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        width[blockIdx.x] = most;
+        if (sum) atomicAdd(nnz, (unsigned long long)sum);
+    }
 }
 
 // The entries of each slice column by column (entry k of row 32 sl + l at
-// ptr[sl] + 32 k + l), each row in increasing column order, padded with zero weights
-// on the row's own column. Weights are stored in FP32 in both precisions (the SpMV
-// works in FP32 per entry); the Jacobi inverse diagonal is taken from the stored
-// weights, so the stored matrix has exactly zero row sums.
-__global__ void sell_fill_kernel(const int32_t* __restrict__ fcnt, const int32_t* __restrict__ fcol,
-                                 const double* __restrict__ fval, int64_t N, int64_t nslice,
-                                 const int64_t* __restrict__ ptr, int32_t* __restrict__ col,
-                                 float* __restrict__ val, double* __restrict__ dinv) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t sl = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < nslice;
-         sl += nw) {
-        const int64_t i = sl * 32 + lane;
-        const int64_t base = ptr[sl] + lane;
-        const int w = (int)((ptr[sl + 1] - ptr[sl]) >> 5);
-        int k = 0;
-        double diag = 0.0;
-        if (i < N) {
-            const int n = fcnt[i];
-            for (int t = 0; t < n && k < w; t++) {
-                const double v = sym_value(fcnt, fcol, fval, i, t);
-                if (!(v > 0.0)) continue;
-                const float vt = (float)v;
-                const int32_t c = fcol[i * FCAP + t];
-                // insertion by column: entry k of neighbouring rows then lies near the
-                // same stencil direction, so the gathers of a warp share cache lines
-                int b = k;
-                for (; b > 0; b--) {
-                    const int32_t cb = col[base + 32 * (int64_t)(b - 1)];
-                    if (cb <= c) break;
-                    col[base + 32 * (int64_t)b] = cb;
-                    val[base + 32 * (int64_t)b] = val[base + 32 * (int64_t)(b - 1)];
-                }
-                col[base + 32 * (int64_t)b] = c;
-                val[base + 32 * (int64_t)b] = vt;
-                diag += (double)vt;
-                k++;
-            }
-            dinv[i] = diag > 0.0 ? 1.0 / diag : 0.0;
-        }
+// ptr[sl] + 32 k + l), each row in increasing column order (entry k of neighbouring rows
+// then lies near the same stencil direction, so the gathers of a warp share cache lines),
+// padded with zero weights on the row's own column. Weights are stored in FP32 in both
+// precisions (the SpMV works in FP32 per entry); the Jacobi inverse diagonal is taken from
+// the stored weights, summed in facet order, so the stored matrix has exactly zero row
+// sums. Blocks and warps as in sell_count_kernel; a lane's rank among the kept columns is
+// its entry.
+__global__ void __launch_bounds__(CG_THREADS)
+    sell_fill_kernel(const int32_t* __restrict__ fcnt, const int32_t* __restrict__ fcol,
+                     const double* __restrict__ fval, int64_t N, const int64_t* __restrict__ ptr,
+                     int32_t* __restrict__ col, float* __restrict__ val,
+                     double* __restrict__ dinv) {
+    __shared__ float wt[32][33];  // weights by row and facet, zero where not kept
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t sl = blockIdx.x;
+    const int64_t p0 = ptr[sl];
+    const int w = (int)((ptr[sl + 1] - p0) >> 5);
+    for (int q = 0; q < SELL_ROWS; q++) {
+        const int row = warp * SELL_ROWS + q;
+        const int64_t i = sl * 32 + row, base = p0 + row;
         const int32_t self = i < N ? (int32_t)i : 0;
-        for (; k < w; k++) {
+        const int n = i < N ? fcnt[i] : 0;
+        int kept = 0;
+        if (n > 32) {  // rare: the row in lane 0, serially (insertion by column)
+            if (lane == 0) {
+                double diag = 0.0;
+                for (int t = 0; t < n && kept < w; t++) {
+                    const double v = sym_value(fcnt, fcol, fval, i, t);
+                    if (!(v > 0.0)) continue;
+                    const float vt = (float)v;
+                    const int32_t c = fcol[i * FCAP + t];
+                    int b = kept;
+                    for (; b > 0; b--) {
+                        const int32_t cb = col[base + 32 * (int64_t)(b - 1)];
+                        if (cb <= c) break;
+                        col[base + 32 * (int64_t)b] = cb;
+                        val[base + 32 * (int64_t)b] = val[base + 32 * (int64_t)(b - 1)];
+                    }
+                    col[base + 32 * (int64_t)b] = c;
+                    val[base + 32 * (int64_t)b] = vt;
+                    diag += (double)vt;
+                    kept++;
+                }
+                dinv[i] = diag > 0.0 ? 1.0 / diag : 0.0;
+            }
+            kept = __shfl_sync(FULLMASK, kept, 0);
+        } else {
+            const RowSym r = row_sym_warp(fcnt, fcol, fval, i, n, lane);
+            const uint32_t km = __ballot_sync(FULLMASK, r.keep);
+            kept = __popc(km);
+            int rank = 0;
+            for (uint32_t m = km; m; m &= m - 1)
+                if (__shfl_sync(FULLMASK, r.j, __ffs(m) - 1) < r.j) rank++;
+            if (r.keep) {
+                col[base + 32 * (int64_t)rank] = r.j;
+                val[base + 32 * (int64_t)rank] = (float)r.v;
+            }
+            wt[row][lane] = r.keep ? (float)r.v : 0.f;
+        }
+        for (int k = kept + lane; k < w; k += 32) {
             col[base + 32 * (int64_t)k] = self;
             val[base + 32 * (int64_t)k] = 0.f;
+        }
+    }
+    __syncthreads();
+    const int64_t i = sl * 32 + lane;
+    if (warp == 0 && i < N) {
+        const int n = fcnt[i];
+        if (n <= 32) {
+            double diag = 0.0;
+            for (int t = 0; t < n; t++) diag += (double)wt[lane][t];
+            dinv[i] = diag > 0.0 ? 1.0 / diag : 0.0;
         }
     }
 }
@@ -534,10 +603,10 @@ __global__ void partial_sum_kernel(const double* __restrict__ part, int nb, int 
 int sell_build(DeviceState& d, int64_t* entries, int64_t* offdiag, cudaStream_t s) {
     const int64_t N = d.N;
     const int64_t nslice = (N + 31) / 32;
-    const int nb = 8 * num_sms();
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(d.scal + 40);
     SDOT_CUDA_TRY(cudaMemsetAsync(cnt, 0, 8, s));
-    sell_count_kernel<<<nb, CG_THREADS, 0, s>>>(d.fcnt, d.fcol, d.fval, N, nslice, d.sell_w, cnt);
+    sell_count_kernel<<<(unsigned)nslice, CG_THREADS, 0, s>>>(d.fcnt, d.fcol, d.fval, N, d.sell_w,
+                                                              cnt);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     SDOT_CUDA_TRY(cudaMemsetAsync(d.sell_w + nslice, 0, 4, s));
@@ -560,12 +629,11 @@ __global__ void scale_ptr_kernel(int64_t* __restrict__ ptr, int64_t n) {
 int sell_fill(DeviceState& d, cudaStream_t s) {
     const int64_t N = d.N;
     const int64_t nslice = (N + 31) / 32;
-    const int nb = 8 * num_sms();
     scale_ptr_kernel<<<(unsigned)((nslice + 1 + 255) / 256), 256, 0, s>>>(d.sell_ptr, nslice + 1);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
-    sell_fill_kernel<<<nb, CG_THREADS, 0, s>>>(d.fcnt, d.fcol, d.fval, N, nslice, d.sell_ptr,
-                                               d.sell_col, d.sell_val, d.dinv);
+    sell_fill_kernel<<<(unsigned)nslice, CG_THREADS, 0, s>>>(d.fcnt, d.fcol, d.fval, N, d.sell_ptr,
+                                                             d.sell_col, d.sell_val, d.dinv);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     return SDOT_OK;
