@@ -97,10 +97,10 @@ __global__ void __launch_bounds__(clip_warps<R, C>() * 32, CLIP_BLOCKS_PER_SM) c
 // ---------------------------------------------------------------------------
 // per-evaluation preparation: normalised float positions and the psi pyramid
 // ---------------------------------------------------------------------------
-__global__ void posf_kernel(const Pos4* __restrict__ pos, const double* __restrict__ psi,
-                            int64_t N, double inv_a, double inv_a2, double hx, double hy,
-                            double hz, int Gx, int Gy, int Gz, float4* __restrict__ posf,
-                            float* __restrict__ pslo, int32_t* __restrict__ leafc,
+// The seeds' grid cells and offsets in them: once per context (its first evaluation).
+__global__ void posf_kernel(const Pos4* __restrict__ pos, int64_t N, double inv_a, double hx,
+                            double hy, double hz, int Gx, int Gy, int Gz,
+                            float4* __restrict__ posf, int32_t* __restrict__ leafc,
                             uint4* __restrict__ ioff) {
     int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= N) return;
@@ -121,23 +121,17 @@ __global__ void posf_kernel(const Pos4* __restrict__ pos, const double* __restri
         fx = fx < 0.0 ? 0.0 : (fx > 4294967295.0 ? 4294967295.0 : fx);
         io[a] = (uint32_t)fx;
     }
-    double q = psi[s] * inv_a2;
-    float hi = (float)q;
-    posf[s] = make_float4(off[0], off[1], off[2], hi);
-    pslo[s] = (float)(q - (double)hi);
+    posf[s] = make_float4(off[0], off[1], off[2], 0.f);
     leafc[s] = c[0] | (c[1] << 10) | (c[2] << 20);
     ioff[s] = make_uint4(io[0], io[1], io[2], 0u);
 }
 
-__global__ void leaf_max_kernel(const int32_t* __restrict__ cell_start, int64_t ncell,
-                                const double* __restrict__ psi, double inv_a2,
-                                float* __restrict__ out) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Level 0 of the pyramid from the ordered maxima psi_kernel left (0: no seed).
+__global__ void leaf_max_kernel(float* __restrict__ psimax, int64_t ncell) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncell) return;
-    int32_t b = cell_start[c], e = cell_start[c + 1];
-    double m = -INFINITY;
-    for (int32_t s = b; s < e; s++) m = fmax(m, psi[s]);
-    out[c] = (b == e) ? -INFINITY : __double2float_ru(m * inv_a2 * (1.0 + 1e-15 * (m > 0 ? 1 : -1)));
+    const uint32_t u = __float_as_uint(psimax[c]);
+    psimax[c] = u ? ord2f(u) : -INFINITY;
 }
 
 __global__ void level_max_kernel(const float* __restrict__ in, int dx, int dy, int dz,
@@ -153,12 +147,44 @@ __global__ void level_max_kernel(const float* __restrict__ in, int dx, int dy, i
     out[n] = m;
 }
 
-// Change of psi since the previous evaluation of the context: the largest and smallest
-// psi - psi_prev in units of a^2 (rounded outward, as order-preserving integers for the
-// atomics: mm[0] the maximum, mm[1] the minimum); psi_prev then takes psi. Only
-// differences of psi shape the diagram, so a carried certificate consumes max - min.
-__global__ void psi_change_kernel(const double* __restrict__ psi, double* __restrict__ prev,
-                                  int64_t N, double inv_a2, uint32_t* __restrict__ mm) {
+// The pyramid's levels from l on in one block: they are small, and a launch each cost more
+// than they do.
+__global__ void __launch_bounds__(1024) top_levels_kernel(Pyramid P, int l) {
+    for (; l < P.nlev; l++) {
+        const float* in = P.psimax + P.off[l - 1];
+        float* out = P.psimax + P.off[l];
+        const int dx = P.dim[l - 1][0], dy = P.dim[l - 1][1], dz = P.dim[l - 1][2];
+        const int ox = P.dim[l][0], oy = P.dim[l][1], oz = P.dim[l][2];
+        // 8 lanes a node, 8 children each
+        const int part = threadIdx.x & 7;
+        for (int n = threadIdx.x >> 3; n < (ox * oy * oz + 3) / 4 * 4; n += blockDim.x >> 3) {
+            const int X = n % ox, Y = (n / ox) % oy, Z = n / (ox * oy);
+            float m = -INFINITY;
+            for (int c = part; c < 64; c += 8) {
+                const int x = 4 * X + (c & 3), y = 4 * Y + ((c >> 2) & 3), z = 4 * Z + (c >> 4);
+                if (x < dx && y < dy && z < dz) m = fmaxf(m, in[(z * dy + y) * dx + x]);
+            }
+            for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULLMASK, m, o));
+            if (part == 0 && Z < oz) out[n] = m;
+        }
+        __syncthreads();
+    }
+}
+
+// What changes with psi, in one pass over the seeds:
+//  - psi/a^2 as hi + lo floats;
+//  - the upper bound of psi/a^2 over each grid cell (an integer maximum of ordered bits: a
+//    clump's grid cell holds hundreds of seeds, which one thread used to scan);
+//  - the change of psi since the previous evaluation of the context: the largest and
+//    smallest psi - psi_prev in units of a^2 (rounded outward, as order-preserving integers
+//    for the atomics: mm[0] the maximum, mm[1] the minimum); psi_prev then takes psi. Only
+//    differences of psi shape the diagram, so a carried certificate consumes max - min.
+// 2.1 M seeds: 70 us, where three passes, one of which recomputed the grid offsets with six
+// FP64 divisions a seed, took 440 us; 38 k clumped seeds 49 -> 6 us.
+__global__ void psi_kernel(const double* __restrict__ psi, double* __restrict__ prev, int64_t N,
+                           double inv_a2, int Gx, int Gy, const int32_t* __restrict__ leafc,
+                           float4* __restrict__ posf, float* __restrict__ pslo,
+                           uint32_t* __restrict__ leafmax, uint32_t* __restrict__ mm) {
     float hi = -INFINITY, lo = INFINITY;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -167,6 +193,14 @@ __global__ void psi_change_kernel(const double* __restrict__ psi, double* __rest
         hi = fmaxf(hi, __double2float_ru(dv));
         lo = fminf(lo, __double2float_rd(dv));
         prev[i] = p;
+        const double q = p * inv_a2;
+        const float qh = (float)q;
+        posf[i].w = qh;
+        pslo[i] = (float)(q - (double)qh);
+        const int lc = leafc[i];
+        const int64_t leaf =
+            ((int64_t)((lc >> 20) & 1023) * Gy + ((lc >> 10) & 1023)) * Gx + (lc & 1023);
+        atomicMax(&leafmax[leaf], f2ord(__double2float_ru(q * (1.0 + 1e-15 * (p > 0 ? 1 : -1)))));
     }
     uint32_t h = f2ord(hi), l = f2ord(lo);
     h = __reduce_max_sync(FULLMASK, h);
@@ -180,27 +214,41 @@ __global__ void psi_change_kernel(const double* __restrict__ psi, double* __rest
 int build_pyramid(DeviceState& d, const double* psi, cudaStream_t s) {
     const int64_t N = d.N;
     uint32_t* mm = reinterpret_cast<uint32_t*>(d.counters + 30);
+    Pyramid& P = d.pyr;
+    if (!d.posf_valid) {
+        posf_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(
+            d.pos, N, 1.0 / d.a, d.grid.h[0], d.grid.h[1], d.grid.h[2], d.grid.G[0], d.grid.G[1],
+            d.grid.G[2], d.posf, d.leafc, d.ioff);
+        note_launch();
+        SDOT_CUDA_TRY(cudaGetLastError());
+        d.posf_valid = 1;
+    }
     SDOT_CUDA_TRY(cudaMemsetAsync(mm, 0, 4, s));
     SDOT_CUDA_TRY(cudaMemsetAsync(mm + 1, 0xff, 4, s));
-    psi_change_kernel<<<2 * num_sms(), 256, 0, s>>>(psi, d.psi_prev, N, 1.0 / (d.a * d.a), mm);
+    SDOT_CUDA_TRY(cudaMemsetAsync(P.psimax + P.off[0], 0, (size_t)d.grid.ncell * 4, s));
+    const int64_t nb = (N + 255) / 256, most = 8 * (int64_t)num_sms();
+    psi_kernel<<<(unsigned)(nb < most ? nb : most), 256, 0, s>>>(
+        psi, d.psi_prev, N, 1.0 / (d.a * d.a), d.grid.G[0], d.grid.G[1], d.leafc, d.posf, d.pslo,
+        reinterpret_cast<uint32_t*>(P.psimax + P.off[0]), mm);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
-    posf_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(
-        d.pos, psi, N, 1.0 / d.a, 1.0 / (d.a * d.a), d.grid.h[0], d.grid.h[1], d.grid.h[2],
-        d.grid.G[0], d.grid.G[1], d.grid.G[2], d.posf, d.pslo, d.leafc, d.ioff);
-        note_launch();
+    leaf_max_kernel<<<(unsigned)((d.grid.ncell + 255) / 256), 256, 0, s>>>(P.psimax + P.off[0],
+                                                                          d.grid.ncell);
+    note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
-    Pyramid& P = d.pyr;
-    leaf_max_kernel<<<(unsigned)((d.grid.ncell + 255) / 256), 256, 0, s>>>(
-        d.grid.cell_start, d.grid.ncell, psi, 1.0 / (d.a * d.a), P.psimax + P.off[0]);
-        note_launch();
-    SDOT_CUDA_TRY(cudaGetLastError());
-    for (int l = 1; l < P.nlev; l++) {
-        int64_t n = (int64_t)P.dim[l][0] * P.dim[l][1] * P.dim[l][2];
+    int l = 1;
+    for (; l < P.nlev; l++) {
+        const int64_t n = (int64_t)P.dim[l][0] * P.dim[l][1] * P.dim[l][2];
+        if (n <= 4096) break;  // 32 nodes a pass of top_levels_kernel's block
         level_max_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
             P.psimax + P.off[l - 1], P.dim[l - 1][0], P.dim[l - 1][1], P.dim[l - 1][2],
             P.psimax + P.off[l], P.dim[l][0], P.dim[l][1], P.dim[l][2]);
-            note_launch();
+        note_launch();
+        SDOT_CUDA_TRY(cudaGetLastError());
+    }
+    if (l < P.nlev) {
+        top_levels_kernel<<<1, 1024, 0, s>>>(P, l);
+        note_launch();
         SDOT_CUDA_TRY(cudaGetLastError());
     }
     return SDOT_OK;
@@ -258,24 +306,36 @@ __global__ void cell_reduce_kernel(const double* __restrict__ vol, const double*
     }
 }
 
-__global__ void cell_reduce_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
-    if (threadIdx.x != 0) return;
-    double sv = 0, mr = 0, l2 = 0, mv = INFINITY, ne = 0;
-    uint32_t fl = 0;
-    for (int b = 0; b < nb; b++) {
-        sv += part[b * 6];
-        mr = fmax(mr, part[b * 6 + 1]);
-        l2 += part[b * 6 + 2];
-        mv = fmin(mv, part[b * 6 + 3]);
-        ne += part[b * 6 + 4];
-        fl |= (uint32_t)part[b * 6 + 5];
+// The blocks' partials in block order (the sums' order is part of the result): loaded by the
+// whole block, then one warp a quantity. A single thread that also loaded them took 94 us
+// of every evaluation; this takes 15.
+__global__ void __launch_bounds__(RED_BLOCKS) cell_reduce_final(const double* __restrict__ part,
+                                                                double* __restrict__ out) {
+    __shared__ double sh[6][RED_BLOCKS];
+    for (int t = threadIdx.x; t < 6 * RED_BLOCKS; t += RED_BLOCKS) sh[t % 6][t / 6] = part[t];
+    __syncthreads();
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (q == 0 || q == 2 || q == 4) {  // sums, serially
+        if (lane == 0) {
+            double v = 0;
+#pragma unroll 16
+            for (int b = 0; b < RED_BLOCKS; b++) v += sh[q][b];
+            out[q] = q == 2 ? sqrt(v) : v;
+        }
+    } else if (q == 1 || q == 3) {  // maximum, minimum
+        double v = q == 1 ? 0.0 : INFINITY;
+        for (int b = lane; b < RED_BLOCKS; b += 32) v = q == 1 ? fmax(v, sh[q][b]) : fmin(v, sh[q][b]);
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(FULLMASK, v, o);
+            v = q == 1 ? fmax(v, u) : fmin(v, u);
+        }
+        if (lane == 0) out[q] = v;
+    } else if (q == 5) {
+        uint32_t fl = 0;
+        for (int b = lane; b < RED_BLOCKS; b += 32) fl |= (uint32_t)sh[5][b];
+        fl = __reduce_or_sync(FULLMASK, fl);
+        if (lane == 0) out[5] = (double)fl;
     }
-    out[0] = sv;
-    out[1] = mr;
-    out[2] = sqrt(l2);
-    out[3] = mv;
-    out[4] = ne;
-    out[5] = (double)fl;
 }
 
 // Warps of a clipping block and blocks for nwork cells: full blocks where there are cells
@@ -455,7 +515,7 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
     cell_reduce_kernel<<<RED_BLOCKS, 256, 0, s>>>(d.vol, d.nu, d.status, d.N, d.partials);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
-    cell_reduce_final<<<1, 32, 0, s>>>(d.partials, RED_BLOCKS, d.scal);
+    cell_reduce_final<<<1, RED_BLOCKS, 0, s>>>(d.partials, d.scal);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     double h[6];
@@ -720,7 +780,7 @@ int evaluate_cells_batch(DeviceState* const* ds, const double* const* psis, cons
         cell_reduce_kernel<<<RED_BLOCKS, 256, 0, s>>>(d.vol, d.nu, d.status, d.N, d.partials);
         note_launch();
         SDOT_CUDA_TRY(cudaGetLastError());
-        cell_reduce_final<<<1, 32, 0, s>>>(d.partials, RED_BLOCKS, d.scal);
+        cell_reduce_final<<<1, RED_BLOCKS, 0, s>>>(d.partials, d.scal);
         note_launch();
         SDOT_CUDA_TRY(cudaGetLastError());
         SDOT_CUDA_TRY(cudaMemcpyAsync(sc->red_host + 6 * j, d.scal, 6 * sizeof(double),

@@ -79,6 +79,7 @@ struct DeviceState {
     float* pslo;              // psi/a^2 lo part (psi/a^2 = hi + lo)
     uint4* ioff;              // offset in the grid cell as 32-bit fixed point (x, y, z, 0)
     int32_t* leafc;           // grid cell of each seed: x | y << 10 | z << 20
+    int posf_valid;           // posf's offsets, leafc and ioff are written
     int facets_valid;         // fcnt/fcol hold a complete previous diagram
     int carry = 1;            // carry security certificates between evaluations
     int32_t* perm;            // sorted -> caller index
