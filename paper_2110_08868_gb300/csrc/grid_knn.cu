@@ -3,8 +3,8 @@
 // The seeds are binned into a G^3 grid of cells of ~seeds_per_leaf seeds, sorted by
 // cell (counting sort; ties inside a cell by caller index, so the order is
 // deterministic) and kept in that order on the device for every later kernel.
-// Each query walks rings of grid cells until its k-th distance is below the distance
-// to the first unvisited ring. The distance key is (d^2, caller index) with
+// Each query takes shells of grid cells until its k-th distance is below the distance
+// to the first unvisited shell. The distance key is (d^2, caller index) with
 // d^2 = (dx*dx + dy*dy) + dz*dz of the minimum-image difference, evaluated with
 // explicit round-to-nearest products and sums (no FMA) so that it is bit-identical
 // to a plain IEEE binary64 evaluation.
@@ -406,10 +406,10 @@ __device__ __noinline__ void knn_exact(const Pos4* __restrict__ pos,
     }
 }
 
-// Grid-local FP32 offsets of every seed (in units of the grid cell) and its grid cell,
-// for the FP32 pass of the search.
+// Grid-local FP32 offsets of every seed (in units of the grid cell) and its grid cell
+// (x | y << 10 | z << 20, in w's bits), for the FP32 pass of the search.
 __global__ void knn_prep_kernel(const Pos4* __restrict__ pos, int64_t N, KnnParams p,
-                                float4* __restrict__ off, int32_t* __restrict__ cellc) {
+                                float4* __restrict__ off) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= N) return;
     const Pos4 y = pos[t];
@@ -422,33 +422,258 @@ __global__ void knn_prep_kernel(const Pos4* __restrict__ pos, int64_t N, KnnPara
         c[a] = cc;
         o[a] = (float)((xs[a] - cc * p.h[a]) / p.h[a]);
     }
-    off[t] = make_float4(o[0], o[1], o[2], 0.f);
-    cellc[t] = c[0] | (c[1] << 10) | (c[2] << 20);
+    off[t] = make_float4(o[0], o[1], o[2], __int_as_float(c[0] | (c[1] << 10) | (c[2] << 20)));
 }
 
-// k nearest seeds of every query. A first pass in FP32 keeps the K + 8 smallest
-// approximate squared distances (grid-cell difference plus FP32 offset difference, in
-// grid-cell units, minimum image); its error is below Delta = 1e-5 (F_k + 1) for
-// distances of a few grid cells, so every seed of the exact top k has an approximate
-// key <= tau = F_k + 2 Delta (F_k: the k-th approximate key). The rings stop once the
-// unvisited seeds are beyond tau + Delta. The entries <= tau then get the exact FP64 key
-// (no FMA, ties by caller index) and are ranked exactly. If the K + 8 entries do not
-// all fit below tau (many near ties, as on a lattice), the query takes the exact
-// search instead. FAST = false (k > 24, where the unrolled lists would cost more
-// registers than they save): the exact search for every query.
-template <int K, bool FAST>
-__global__ void __launch_bounds__(128) knn_kernel(const Pos4* __restrict__ pos,
-                                                  const float4* __restrict__ off,
-                                                  const int32_t* __restrict__ cellc,
-                                                  const int32_t* __restrict__ cell_start,
-                                                  KnnParams p, int32_t* __restrict__ knn,
-                                                  double* __restrict__ d2k,
-                                                  int* __restrict__ flags) {
-    constexpr int K2 = K + 8;
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// k nearest seeds of every query, one warp a query.
+//
+// An FP32 pass keeps the seeds that may be among the nearest: approximate squared distances
+// (grid-cell difference plus FP32 offset difference, in grid-cell units, minimum image),
+// whose error is below Delta = 1e-5 (F_k + 1) for distances of a few grid cells, so every
+// seed of the exact top k has an approximate key <= tau = F_k + 2 Delta (F_k: the k-th
+// approximate key so far). The block of 3^3 grid cells around the query, then the shells
+// beyond it, until the unvisited seeds are beyond tau + Delta. A row of grid cells along x
+// is one run of the sorted order (the two ends of a row inside a shell are two), so 32
+// lanes test 32 seeds at a time; the ones within tau are appended to a buffer of the warp,
+// which is cut back to tau when it fills up. The entries left get the exact FP64 key (no
+// FMA, ties by caller index) and each counts the entries before it: its place.
+// What does not fit (shells that would wrap, more near ties than the buffer holds, as on a
+// lattice with a large k) goes to a queue for the exact search.
+//
+// A thread a query with a sorted list in registers was bound by its serial chain (168
+// registers, 12 warps an SM): 912,673 seeds, k = 24: 10.8 -> 2.6 ms; 4913 seeds, where 39
+// blocks were all there was: 250 -> 27 us.
+constexpr int KNN_WARPS = 8;   // queries of a block
+constexpr int KNN_BUF = 128;   // buffer entries, 4 a lane
+constexpr int KNN_FINAL = 96;  // entries that are ranked exactly, 3 a lane
+
+struct KnnBuf {
+    float key[KNN_BUF];
+    int32_t s[KNN_BUF];
+    unsigned long long d[KNN_FINAL];  // exact keys, as ordered bits
+    int32_t o[KNN_FINAL];             // caller index
+};
+
+// Cut the buffer of n entries back to those <= tau; returns their number and tau (FLT_MAX
+// while there are fewer than k). The k-th smallest key by bisection on the keys' bits
+// (ordered, as they are not negative); it ends as soon as a pivot leaves exactly k below.
+__device__ __forceinline__ int knn_prune(KnnBuf& B, int n, int k, float& tau, int lane) {
+    if (n < k) return n;
+    uint32_t v[4];
+    int32_t s[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+        const int t = lane + 32 * e;
+        v[e] = t < n ? __float_as_uint(B.key[t]) : 0xffffffffu;
+        s[e] = t < n ? B.s[t] : -1;
+    }
+    uint32_t lo = __reduce_min_sync(0xffffffffu, min(min(v[0], v[1]), min(v[2], v[3])));
+    uint32_t mx = 0;
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+        if (v[e] != 0xffffffffu) mx = max(mx, v[e]);
+    uint32_t hi = __reduce_max_sync(0xffffffffu, mx);
+    while (lo < hi) {  // at most 32 steps; count(<= hi) >= k throughout
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        int c = 0;
+#pragma unroll
+        for (int e = 0; e < 4; e++) c += v[e] <= mid ? 1 : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c >= k) hi = mid;
+        else lo = mid + 1;
+        if (c == k) break;
+    }
+    mx = 0;
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+        if (v[e] <= hi) mx = max(mx, v[e]);
+    const float Fk = __uint_as_float(__reduce_max_sync(0xffffffffu, mx));
+    tau = Fk + 2.f * (1e-5f * (Fk + 1.f));
+    const uint32_t tb = __float_as_uint(tau);
+    int m = 0;
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+        const uint32_t b = __ballot_sync(0xffffffffu, v[e] <= tb);
+        if (v[e] <= tb) {
+            const int at = m + __popc(b & ((1u << lane) - 1u));
+            B.key[at] = __uint_as_float(v[e]);
+            B.s[at] = s[e];
+        }
+        m += __popc(b);
+    }
+    __syncwarp();
+    return m;
+}
+
+__global__ void __launch_bounds__(KNN_WARPS * 32)
+    knn_kernel(const Pos4* __restrict__ pos, const float4* __restrict__ off,
+               const int32_t* __restrict__ cell_start, KnnParams p, int32_t* __restrict__ knn,
+               double* __restrict__ d2k, int* __restrict__ flags, int32_t* __restrict__ rest,
+               int32_t* __restrict__ nrest) {
+    __shared__ KnnBuf bufs[KNN_WARPS];
+    const int lane = threadIdx.x & 31;
+    KnnBuf& B = bufs[threadIdx.x >> 5];
+    const int64_t q = (int64_t)blockIdx.x * KNN_WARPS + (threadIdx.x >> 5);
     if (q >= p.N) return;
     const int k = p.k;
-    if (!FAST) {  // large k: the exact search only
+    const float4 oi = off[q];
+    const int lc = __float_as_int(oi.w);
+    const int c[3] = {lc & 1023, (lc >> 10) & 1023, (lc >> 20) & 1023};
+    const float G[3] = {(float)p.G[0], (float)p.G[1], (float)p.G[2]};
+    // grid cells are near-cubic; distances in units of the x cell size
+    const float sy = (float)(p.h[1] / p.h[0]), sz = (float)(p.h[2] / p.h[0]);
+    const float m = fminf(fminf(fminf(oi.x, 1.f - oi.x), fminf(oi.y, 1.f - oi.y) * sy),
+                          fminf(oi.z, 1.f - oi.z) * sz);
+    const int Gmin = min(p.G[0], min(p.G[1], p.G[2]));
+    float tau = FLT_MAX;
+    int n = 0;
+    bool ok = false, full = false;
+    for (int r = 1; 2 * r + 1 <= Gmin && !full; r++) {
+        const int w = 2 * r + 1, rows = w * w;
+        for (int base = 0; base < rows && !full; base += 32) {
+            // this lane's row of grid cells: one run, or two
+            const int row = base + lane;
+            int32_t s0 = 0, s1 = 0;
+            int n0 = 0, n1 = 0;
+            if (row < rows) {
+                const int rz = row / w, ry = row - rz * w;
+                int cy = c[1] + ry - r, cz = c[2] + rz - r;
+                if (cy < 0) cy += p.G[1];
+                else if (cy >= p.G[1]) cy -= p.G[1];
+                if (cz < 0) cz += p.G[2];
+                else if (cz >= p.G[2]) cz -= p.G[2];
+                const int32_t* cs = cell_start + ((int64_t)cz * p.G[1] + cy) * p.G[0];
+                int X0 = c[0] - r, X1 = c[0] + r;
+                // r = 1 takes the whole block, later shells only their own cells
+                const bool whole = r == 1 || ry == 0 || ry == w - 1 || rz == 0 || rz == w - 1;
+                if (whole) {
+                    if (X0 < 0) {
+                        X0 += p.G[0];
+                        X1 += p.G[0];
+                    }
+                    s0 = cs[X0];
+                    n0 = cs[min(X1, p.G[0] - 1) + 1] - s0;
+                    if (X1 >= p.G[0]) {
+                        s1 = cs[0];
+                        n1 = cs[X1 - p.G[0] + 1] - s1;
+                    }
+                } else {
+                    if (X0 < 0) X0 += p.G[0];
+                    if (X1 >= p.G[0]) X1 -= p.G[0];
+                    s0 = cs[X0];
+                    n0 = cs[X0 + 1] - s0;
+                    s1 = cs[X1];
+                    n1 = cs[X1 + 1] - s1;
+                }
+            }
+            const int nn = n0 + n1;
+            int incl = nn;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            const int excl = incl - nn;
+            const int32_t first = s0 - excl, jump = s1 - (s0 + n0);
+            const int split = excl + n0;
+            for (int b = 0; b < total; b += 32) {
+                const int t = b + lane;
+                // the lane owning flattened seed t: the first with incl > t
+                int u = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1) {
+                    const int y = __shfl_sync(0xffffffffu, incl, u + step - 1);
+                    if (y <= t) u += step;
+                }
+                int32_t s = t + __shfl_sync(0xffffffffu, first, u);
+                const int sp = __shfl_sync(0xffffffffu, split, u);
+                const int32_t jq = __shfl_sync(0xffffffffu, jump, u);
+                if (t >= sp) s += jq;
+                float d2 = FLT_MAX;
+                if (t < total && s != (int32_t)q) {
+                    const float4 oj = off[s];
+                    const int lj = __float_as_int(oj.w);
+                    const int cj[3] = {lj & 1023, (lj >> 10) & 1023, (lj >> 20) & 1023};
+                    const float dd[3] = {oj.x - oi.x, oj.y - oi.y, oj.z - oi.z};
+                    float dx[3];
+#pragma unroll
+                    for (int a = 0; a < 3; a++) {
+                        int dc = cj[a] - c[a];
+                        if (2 * dc > p.G[a]) dc -= p.G[a];
+                        else if (2 * dc < -p.G[a]) dc += p.G[a];
+                        dx[a] = (float)dc + dd[a];
+                        if (dx[a] > 0.5f * G[a]) dx[a] -= G[a];
+                        else if (dx[a] < -0.5f * G[a]) dx[a] += G[a];
+                    }
+                    dx[1] *= sy;
+                    dx[2] *= sz;
+                    d2 = dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2];
+                }
+                const bool keep = d2 <= tau && d2 < FLT_MAX;
+                const uint32_t km = __ballot_sync(0xffffffffu, keep);
+                if (!km) continue;
+                if (keep) {
+                    const int at = n + __popc(km & ((1u << lane) - 1u));
+                    B.key[at] = d2;
+                    B.s[at] = s;
+                }
+                n += __popc(km);
+                __syncwarp();
+                if (n > KNN_BUF - 32) {
+                    n = knn_prune(B, n, k, tau, lane);
+                    if (n > KNN_BUF - 32) {  // too many near ties
+                        full = true;
+                        break;
+                    }
+                }
+            }
+        }
+        if (full) break;
+        n = knn_prune(B, n, k, tau, lane);
+        if (n < k) continue;
+        // every unvisited seed lies at least r + m cell sizes away; tau's Delta is (tau -
+        // F_k) / 2
+        const float bound = (float)r * fminf(1.f, fminf(sy, sz)) + m;
+        if (tau + 1e-5f * (tau + 1.f) < bound * bound * (1.f - 1e-6f)) {
+            ok = true;
+            break;
+        }
+    }
+    if (!ok || n > KNN_FINAL) {
+        if (lane == 0) rest[atomicAdd(nrest, 1)] = (int32_t)q;
+        return;
+    }
+    // exact keys, then each entry's place among them
+    const Pos4 yi = pos[q];
+    for (int e = lane; e < n; e += 32) {
+        const Pos4 yj = pos[B.s[e]];
+        B.d[e] = (unsigned long long)__double_as_longlong(dist2_exact(yi, yj, p));
+        B.o[e] = (int)yj.w;
+    }
+    __syncwarp();
+    for (int e = lane; e < n; e += 32) {
+        const unsigned long long d = B.d[e];
+        const int o = B.o[e];
+        int place = 0;
+        for (int u = 0; u < n; u++) place += B.d[u] < d || (B.d[u] == d && B.o[u] < o) ? 1 : 0;
+        if (place < k) knn[q * k + place] = B.s[e];
+        if (place == k - 1) d2k[q] = __longlong_as_double((long long)d);
+        if (place == 0 && d == 0ull) atomicOr(flags, 1);  // duplicate position
+    }
+}
+
+// the queries knn_kernel left, one thread each, by the exact search
+template <int K>
+__global__ void __launch_bounds__(128)
+    knn_rest_kernel(const Pos4* __restrict__ pos, const int32_t* __restrict__ cell_start,
+                    KnnParams p, const int32_t* __restrict__ rest,
+                    const int32_t* __restrict__ nrest, int32_t* __restrict__ knn,
+                    double* __restrict__ d2k, int* __restrict__ flags) {
+    const int k = p.k;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < *nrest;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t q = rest[e];
         TopK<K> top;
         knn_exact<K>(pos, cell_start, p, q, top);
 #pragma unroll
@@ -456,104 +681,9 @@ __global__ void __launch_bounds__(128) knn_kernel(const Pos4* __restrict__ pos,
             if (t < k) knn[q * k + t] = top.s[t];
             if (t == k - 1) d2k[q] = top.d[t];
         }
-        if (top.d[0] == 0.0) atomicOr(flags, 1);
-        if (top.s[0] < 0) atomicOr(flags, 2);
-        return;
+        if (top.d[0] == 0.0) atomicOr(flags, 1);  // duplicate position
+        if (top.s[0] < 0) atomicOr(flags, 2);      // fewer than k other seeds
     }
-    const float4 oi = off[q];
-    const int lc = cellc[q];
-    const int c[3] = {lc & 1023, (lc >> 10) & 1023, (lc >> 20) & 1023};
-    const float G[3] = {(float)p.G[0], (float)p.G[1], (float)p.G[2]};
-    // grid cells are near-cubic; distances in units of the x cell size
-    const float sy = (float)(p.h[1] / p.h[0]), sz = (float)(p.h[2] / p.h[0]);
-    float fd[K2];
-    int fi[K2];
-#pragma unroll
-    for (int t = 0; t < K2; t++) {
-        fd[t] = FLT_MAX;
-        fi[t] = -1;
-    }
-    const float m = fminf(fminf(fminf(oi.x, 1.f - oi.x), fminf(oi.y, 1.f - oi.y) * sy),
-                          fminf(oi.z, 1.f - oi.z) * sz);
-    const int Gmin = min(p.G[0], min(p.G[1], p.G[2]));
-    bool ok = false;
-    float tau = FLT_MAX;
-    for (int r = 0;; r++) {
-        if (2 * r + 1 > Gmin) break;  // rings would wrap: exact search
-        for (int oz = -r; oz <= r; oz++) {
-            const int cz = ((c[2] + oz) % p.G[2] + p.G[2]) % p.G[2];
-            for (int oy = -r; oy <= r; oy++) {
-                const int cy = ((c[1] + oy) % p.G[1] + p.G[1]) % p.G[1];
-                const bool face = (oz == -r || oz == r || oy == -r || oy == r);
-                const int step = (face || r == 0) ? 1 : 2 * r;
-                for (int ox = -r; ox <= r; ox += step) {
-                    const int cx = ((c[0] + ox) % p.G[0] + p.G[0]) % p.G[0];
-                    const int64_t cell = ((int64_t)cz * p.G[1] + cy) * p.G[0] + cx;
-                    const int32_t b = cell_start[cell], e = cell_start[cell + 1];
-                    for (int32_t t = b; t < e; t++) {
-                        if (t == q) continue;
-                        const float4 oj = off[t];
-                        float dx = (float)ox + (oj.x - oi.x);
-                        float dy = (float)oy + (oj.y - oi.y);
-                        float dz = (float)oz + (oj.z - oi.z);
-                        if (dx > 0.5f * G[0]) dx -= G[0];
-                        else if (dx < -0.5f * G[0]) dx += G[0];
-                        if (dy > 0.5f * G[1]) dy -= G[1];
-                        else if (dy < -0.5f * G[1]) dy += G[1];
-                        if (dz > 0.5f * G[2]) dz -= G[2];
-                        else if (dz < -0.5f * G[2]) dz += G[2];
-                        dy *= sy;
-                        dz *= sz;
-                        const float d2 = dx * dx + dy * dy + dz * dz;
-                        if (d2 < fd[K2 - 1]) {
-#pragma unroll
-                            for (int u = K2 - 1; u >= 0; u--) {
-                                if (d2 < fd[u]) {
-                                    const bool sh = u > 0 && d2 < fd[u - 1];
-                                    fd[u] = sh ? fd[u - 1] : d2;
-                                    fi[u] = sh ? fi[u - 1] : t;
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        float Fk = FLT_MAX;
-#pragma unroll
-        for (int t = 0; t < K2; t++)
-            if (t == k - 1) Fk = fd[t];
-        if (Fk == FLT_MAX) continue;
-        const float delta = 1e-5f * (Fk + 1.f);
-        tau = Fk + 2.f * delta;
-        // every unvisited seed lies at least r + m cell sizes away
-        const float bound = fminf((float)r * fminf(1.f, fminf(sy, sz)) + m, 1e30f);
-        if (tau + delta < bound * bound * (1.f - 1e-6f)) {
-            ok = true;
-            break;
-        }
-    }
-    TopK<K> top;
-    if (ok && fd[K2 - 1] <= tau) ok = false;  // too many near ties for the list
-    if (ok) {
-        const Pos4 yi = pos[q];
-        top.init();
-#pragma unroll
-        for (int u = 0; u < K2; u++)
-            if (fd[u] <= tau && fi[u] >= 0) {
-                const Pos4 yj = pos[fi[u]];
-                top.insert(dist2_exact(yi, yj, p), (int)yj.w, fi[u]);
-            }
-    } else {
-        knn_exact<K>(pos, cell_start, p, q, top);
-    }
-#pragma unroll
-    for (int t = 0; t < K; t++) {
-        if (t < k) knn[q * k + t] = top.s[t];
-        if (t == k - 1) d2k[q] = top.d[t];
-    }
-    if (top.d[0] == 0.0) atomicOr(flags, 1);  // duplicate position
-    if (top.s[0] < 0) atomicOr(flags, 2);      // fewer than k other seeds
 }
 
 int build_knn(DeviceState& d, cudaStream_t s, int* dup_flag_host) {
@@ -568,22 +698,26 @@ int build_knn(DeviceState& d, cudaStream_t s, int* dup_flag_host) {
     p.N = d.N;
     p.k = d.k;
     int* flags = (int*)(d.counters + 3);
-    SDOT_CUDA_TRY(cudaMemsetAsync(flags, 0, 4, s));
-    // FP32 grid-local offsets and grid cells: posf and leafc serve as scratch here (the
-    // first Laguerre evaluation rewrites both)
-    const unsigned nb = (unsigned)((d.N + 127) / 128);
-    knn_prep_kernel<<<nb, 128, 0, s>>>(d.pos, d.N, p, d.posf, d.leafc);
+    int32_t* nrest = d.counters + 4;
+    SDOT_CUDA_TRY(cudaMemsetAsync(flags, 0, 8, s));
+    // FP32 grid-local offsets and grid cells: posf serves as scratch here (the first
+    // Laguerre evaluation rewrites it), queue holds the queries for the exact search
+    knn_prep_kernel<<<(unsigned)((d.N + 127) / 128), 128, 0, s>>>(d.pos, d.N, p, d.posf);
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
-#define SDOT_KNN_LAUNCH(KK, F)                                                           \
-    knn_kernel<KK, F><<<nb, 128, 0, s>>>(d.pos, d.posf, d.leafc, d.grid.cell_start, p, \
-                                         d.knn, d.knn_d2k, flags)
-    if (d.k <= 8) SDOT_KNN_LAUNCH(8, true);
-    else if (d.k <= 16) SDOT_KNN_LAUNCH(16, true);
-    else if (d.k <= 24) SDOT_KNN_LAUNCH(24, true);
-    else if (d.k <= 32) SDOT_KNN_LAUNCH(32, false);
-    else SDOT_KNN_LAUNCH(64, false);
-#undef SDOT_KNN_LAUNCH
+    knn_kernel<<<(unsigned)((d.N + KNN_WARPS - 1) / KNN_WARPS), KNN_WARPS * 32, 0, s>>>(
+        d.pos, d.posf, d.grid.cell_start, p, d.knn, d.knn_d2k, flags, d.queue, nrest);
+    note_launch();
+    SDOT_CUDA_TRY(cudaGetLastError());
+    const int64_t rb = (d.N + 127) / 128, most = 4 * (int64_t)num_sms();
+    const unsigned nb = (unsigned)(rb < most ? rb : most);
+#define SDOT_KNN_REST(KK)                                                                    \
+    knn_rest_kernel<KK><<<nb, 128, 0, s>>>(d.pos, d.grid.cell_start, p, d.queue, nrest, d.knn, \
+                                           d.knn_d2k, flags)
+    if (d.k <= 16) SDOT_KNN_REST(16);
+    else if (d.k <= 32) SDOT_KNN_REST(32);
+    else SDOT_KNN_REST(64);
+#undef SDOT_KNN_REST
     note_launch();
     SDOT_CUDA_TRY(cudaGetLastError());
     int h = 0;

@@ -109,16 +109,17 @@ struct DeviceState {
     int32_t* cert_j;          // N * CERT_NEAR
     uint8_t* cert_n;          // N
     double* psi_prev;         // N
-    int32_t* queue;           // N, re-queued cells
+    int32_t* queue;           // N, re-queued cells (kNN build: queries for the exact search)
     int32_t* queue64;         // N, cells for the FP64 re-clip
     int32_t* counters;        // [0] requeue count [1] fp64 count [2] work counter
                               // [3] error flags [4] work counter 2 [5] work counter 3
-                              // [8..24) 64-bit diagnostic work counters
+                              // [7] count of cells not carried [8..24) 64-bit diagnostic
+                              // work counters [25] work counter of the carried pass
     // CSR (sorted order)
     int64_t* row_ptr;         // N + 1
     int32_t* col;             // nnz capacity N * (FCAP + 1)
     double* val;
-    int32_t* rowcnt;          // N (+1 pad)
+    int32_t* rowcnt;          // N (+1 pad); in an evaluation the cells not carried
     // CSR (caller order), built on demand for sdot_laguerre
     int64_t* row_ptr_u;
     int32_t* col_u;
