@@ -2097,124 +2097,6 @@ __device__ __forceinline__ bool process_cell(int slot, const ClipParams& cp, boo
 
 namespace sdot {
 
-// Volume of the polytope (units of a^3), FP64 sum of per-face fan tetrahedra from the
-// centre of the vertices' bounding box, the faces found as in integrate. Every lane
-// gets the value; 0 when a face cycle is broken.
-template <typename R, class C>
-__device__ __noinline__ double poly_volume(int slot, int lane) {
-    Poly<R, C>& P = poly_at<R, C>(slot);
-    constexpr int FPL = (C::MP + 31) / 32;
-    R o[3];
-    {
-        R mn[3] = {R(1e30), R(1e30), R(1e30)}, mxv[3] = {R(-1e30), R(-1e30), R(-1e30)};
-        for (int s2 = lane; s2 < P.nt; s2 += 32) {
-            const R v[3] = {P.vx[s2], P.vy[s2], P.vz[s2]};
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                mn[a] = fmin(mn[a], v[a]);
-                mxv[a] = fmax(mxv[a], v[a]);
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            for (int q = 16; q > 0; q >>= 1) {
-                mn[a] = fmin(mn[a], __shfl_xor_sync(FULLMASK, mn[a], q));
-                mxv[a] = fmax(mxv[a], __shfl_xor_sync(FULLMASK, mxv[a], q));
-            }
-            o[a] = R(0.5) * (mn[a] + mxv[a]);
-        }
-    }
-    const int nt = P.nt, np = P.np;
-    for (int f = lane; f < np; f += 32) P.fend[f] = 0u;
-    __syncwarp();
-    for (int s2 = lane; s2 < nt; s2 += 32) {
-        const uint32_t t = P.tri[s2];
-        atomicAdd(&P.fend[t & 0xff], 1u);
-        atomicAdd(&P.fend[(t >> 8) & 0xff], 1u);
-        atomicAdd(&P.fend[(t >> 16) & 0xff], 1u);
-    }
-    __syncwarp();
-    int fcount[FPL];
-    {
-        uint32_t carry = 0;
-        for (int k = 0; k < FPL; k++) {
-            const int f = lane + 32 * k;
-            const uint32_t c = f < np ? P.fend[f] : 0u;
-            fcount[k] = (int)c;
-            uint32_t incl = c;
-            for (int q = 1; q < 32; q <<= 1) {
-                const uint32_t y = __shfl_up_sync(FULLMASK, incl, q);
-                if (lane >= q) incl += y;
-            }
-            if (f < np) P.fend[f] = carry + incl - c;
-            carry += __shfl_sync(FULLMASK, incl, 31);
-        }
-    }
-    __syncwarp();
-    for (int s2 = lane; s2 < nt; s2 += 32) {
-        const uint32_t t = P.tri[s2];
-        const uint32_t a = t & 0xff, b = (t >> 8) & 0xff, c = (t >> 16) & 0xff;
-        const uint32_t sv = (uint32_t)s2 << 16;
-        P.fent[atomicAdd(&P.fend[a], 1u)] = b | (c << 8) | sv;
-        P.fent[atomicAdd(&P.fend[b], 1u)] = c | (a << 8) | sv;
-        P.fent[atomicAdd(&P.fend[c], 1u)] = a | (b << 8) | sv;
-    }
-    __syncwarp();
-    double vol6 = 0.0;
-    bool ok = true;
-    for (int k = 0; k < FPL; k++) {
-        const int f = lane + 32 * k;
-        const int m = fcount[k];
-        if (f >= np || m == 0) continue;
-        if (m < 3) {
-            ok = false;
-            continue;
-        }
-        const int e0 = (int)P.fend[f] - m;
-        int first = e0;
-        for (int e = e0 + 1; e < e0 + m; e++)
-            if ((P.fent[e] >> 16) < (P.fent[first] >> 16)) first = e;
-        uint32_t ecur = P.fent[first];
-        const uint32_t x0 = ecur & 0xff;
-        V3<R> v0 = vert(P, ecur >> 16);
-        v0.x -= o[0];
-        v0.y -= o[1];
-        v0.z -= o[2];
-        V3<R> vp = v0;
-        R fv6 = 0;
-        for (int step = 1; step < m; step++) {
-            const uint32_t yv = (ecur >> 8) & 0xff;
-            int nxt = -1;
-            for (int e = e0; e < e0 + m; e++)
-                if ((P.fent[e] & 0xff) == yv) {
-                    nxt = e;
-                    break;
-                }
-            if (nxt < 0 || nxt == first) {
-                ok = false;
-                break;
-            }
-            ecur = P.fent[nxt];
-            V3<R> vc = vert(P, ecur >> 16);
-            vc.x -= o[0];
-            vc.y -= o[1];
-            vc.z -= o[2];
-            if (step >= 2) {
-                const R ax = vp.x - v0.x, ay = vp.y - v0.y, az = vp.z - v0.z;
-                const R bx = vc.x - v0.x, by = vc.y - v0.y, bz = vc.z - v0.z;
-                const R cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-                fv6 += v0.x * cx + v0.y * cy + v0.z * cz;
-            }
-            vp = vc;
-        }
-        if (((ecur >> 8) & 0xff) != x0) ok = false;
-        vol6 += (double)fv6;
-    }
-    vol6 = warp_sum(vol6);
-    ok = __all_sync(FULLMASK, ok);
-    return ok ? vol6 / 6.0 : 0.0;
-}
-
 // polytope slot2 <- slot1 (warp-uniform)
 template <typename R, class C>
 __device__ __noinline__ void poly_copy(int slot2, int slot1, int lane) {
