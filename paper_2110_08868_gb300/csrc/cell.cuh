@@ -143,7 +143,7 @@ struct Poly {
 // take a polytope's slot, not its address: through the array the compiler knows that every
 // access is to shared memory. What is the same for a warp (the cell's context, its
 // bounds) is kept there too, once, and not in every lane's stack frame.
-extern __shared__ __align__(16) unsigned char g_polytopes[];
+extern __shared__ __align__(32) unsigned char g_polytopes[];
 template <typename R, class C>
 __device__ __forceinline__ Poly<R, C>& poly_at(int slot) {
     return reinterpret_cast<Poly<R, C>*>(g_polytopes)[slot];
@@ -1741,13 +1741,34 @@ __device__ __noinline__ bool topo_init(int slot, const ClipParams& cp, int nf, i
     }
     ok = __all_sync(FULLMASK, ok);
     if (!ok) return false;
+    if (sizeof(R) == 8) {
+        // the facets' planes in FP32 (the clip's scratch is free): nearly every vertex is far
+        // inside the planes it is not on, which FP32 can say; FP64 decides the rest. The
+        // FP64 tests were 140 instructions at 16 cycles each: FP64 step 45^3
+        // 15.3 -> 14.2 ms, mesh 48^3 to 96^3 12.6 -> 11.9 ms.
+        static_assert(sizeof(float4) * C::MP <= 3 * C::MNEW * sizeof(R) || sizeof(R) == 4,
+                      "the planes share the new vertices");
+        float4* plf = reinterpret_cast<float4*>(P.fx);
+        for (int q = 6 + lane; q < (int)npl; q += 32)
+            plf[q] = make_float4((float)P.pl[q].x, (float)P.pl[q].y, (float)P.pl[q].z,
+                                 (float)P.pl[q].w);
+        __syncwarp();
+    }
 #pragma unroll 1
     for (int s = lane; s < nt; s += 32) {
         const V3<R> v = vert(P, s);
         const uint32_t t = P.tri[s];
         const uint32_t a = t & 0xff, b = (t >> 8) & 0xff, c = (t >> 16) & 0xff;
+        const float fx = (float)v.x, fy = (float)v.y, fz = (float)v.z;
+        const float l1 = fabsf(fx) + fabsf(fy) + fabsf(fz);
         for (uint32_t q = 6; q < npl; q++) {
             if (q == a || q == b || q == c) continue;
+            if (sizeof(R) == 8) {
+                const float4 pf = reinterpret_cast<const float4*>(P.fx)[q];
+                const float tol =
+                    4e-6f * (fabsf(pf.w) + (fabsf(pf.x) + fabsf(pf.y) + fabsf(pf.z)) * l1);
+                if (pf.x * fx + pf.y * fy + pf.z * fz - pf.w < -tol) continue;
+            }
             R sd;
             if (beyond(v, P.pl[q], P.plen[q], sd)) ok = false;
         }
