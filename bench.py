@@ -58,9 +58,9 @@ CG_BYTES_PER_ROW = 124
 CG_BYTES_PER_ENTRY = 8
 # DRAM bytes (read + write) per unit from ncu captures of the current kernels on the
 # clumpy 128^3 box (N = 2,202,087), scaled to a launch by the units it processes (None:
-# not captured since the kernel last changed): the first clipping pass per cell
-# (1.569 + 7.206 GB), one CG iteration (SpMV 402.4 MB + update 162.8 MB) per row
-CLIP_DRAM_PER_CELL = (1.569416e9 + 7.205903e9) / 2202087
+# not captured since the kernel last changed): the first clipping pass per cell, one CG
+# iteration (SpMV 402.4 MB + update 162.8 MB) per row
+CLIP_DRAM_PER_CELL = None
 CG_DRAM_PER_ROW = (385.858560e6 + 16.551168e6 + 123.337216e6 + 39.467264e6) / 2202087
 
 
@@ -408,7 +408,7 @@ def run_native(args, rank, world, local):
     clock_ghz = (clocks["sm_mhz"] or peaks.get("sm_max_mhz", 2070.0)) / 1e3
     peak_tf = N_SM * FP32_LANES_PER_SM * 2 * clock_ghz / 1e3
     achieved_tf = N * FLOP_PER_CELL / (pass1_ms / 1e3) / 1e12
-    kname = "clip_kernel<float,CapS,certify>" if args.precision == "mixed" else \
+    kname = "carry_kernel + clip_kernel<float,CapS,certify>" if args.precision == "mixed" else \
         "clip_kernel<double,CapS,certify>"
     roofline = {"kernel": kname + " (first clipping pass)", "bound": "alu",
                 "launches_timed": len(pass1), "achieved": achieved_tf, "peak": peak_tf,
