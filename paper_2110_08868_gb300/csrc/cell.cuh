@@ -1253,6 +1253,8 @@ __device__ __noinline__ uint32_t traverse(int slot, const ClipParams& cp, int la
 // more than WINDOW_CELLS grid cells or wrap onto itself: the caller then walks the
 // pyramid. (A psimax far above its surroundings, next to a clump, widens the window for
 // every direction, where the pyramid opens only the nodes that need it.)
+// WINDOW_CELLS of 300, 1000, 4000, 16000: first diagram 97^3 147, 115, 114, 113 ms; the first
+// passes of a solve with 105 clumps (929 k cells) 1101, 1087, 1075, 1135 ms.
 enum { WALK_DONE = 0, WALK_STOP = 1, WALK_OTHER = 2 };
 constexpr int WINDOW_CELLS = 1000;
 
