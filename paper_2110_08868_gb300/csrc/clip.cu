@@ -493,8 +493,9 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
     cudaEventRecord(ep2, s);
     int64_t reclipped = cnt[1];
     // pass 3: FP64 re-clip of the cells failing the FP32 checks or over the small
-    // capacity: the small polytope first (its overflows are appended to the same queue),
-    // then the large one for those
+    // capacity: the small polytope first, then the large one for its overflows. Those go to
+    // the re-queue pass's list, which is free by now and holds every cell: the cells of
+    // pass 3 may fill queue64 already, and an overflow is in it a second time.
     if (reclipped > 0) {
         cp.pass = 3;
         cp.work_counter = d.counters + 5;
@@ -502,12 +503,15 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
         cp.nwork = reclipped;
         cp.nwork_dev = nullptr;
         if (precision != SDOT_PREC_FP64) {
+            cp.q64_out = d.queue;
+            cp.q64_cnt = d.counters;
+            SDOT_CUDA_TRY(cudaMemsetAsync(d.counters, 0, sizeof(int32_t), s));
             if ((rc = launch_clip<double, CapS, MODE_FULL>(cp, s))) return rc;
-            SDOT_CUDA_TRY(cudaMemcpyAsync(cnt, d.counters, 8, cudaMemcpyDeviceToHost, s));
+            SDOT_CUDA_TRY(cudaMemcpyAsync(cnt, d.counters, 4, cudaMemcpyDeviceToHost, s));
             SDOT_CUDA_TRY(cudaStreamSynchronize(s));
             cp.work_counter = d.counters + 6;
-            cp.worklist = d.queue64 + reclipped;
-            cp.nwork = (int64_t)cnt[1] - reclipped;
+            cp.worklist = d.queue;
+            cp.nwork = cnt[0];
         }
         if (cp.nwork > 0 && (rc = launch_clip<double, CapL, MODE_FULL>(cp, s))) return rc;
     }

@@ -109,9 +109,10 @@ struct DeviceState {
     int32_t* cert_j;          // N * CERT_NEAR
     uint8_t* cert_n;          // N
     double* psi_prev;         // N
-    int32_t* queue;           // N, re-queued cells (kNN build: queries for the exact search)
-    int32_t* queue64;         // N, cells for the FP64 re-clip
-    int32_t* counters;        // [0] requeue count [1] fp64 count [2] work counter
+    int32_t* queue;           // N, re-queued cells, then the FP64 re-clip's overflows (kNN
+                              // build: queries for the exact search)
+    int32_t* queue64;         // N, cells for the FP64 re-clip, each once
+    int32_t* counters;        // [0] count of queue [1] of queue64 [2] work counter
                               // [3] error flags [4] work counter 2 [5] work counter 3
                               // [7] count of cells not carried [8..24) 64-bit diagnostic
                               // work counters [25] work counter of the carried pass
