@@ -160,12 +160,15 @@ __global__ void __launch_bounds__(SPEC_THREADS)
             const uint32_t live = __ballot_sync(0xffffffffu, bin != INT_MAX);
             if (!live) break;  // larger |n| only from here on
             double p = 0.0;
+            unsigned long long top = 0;  // u >= 0: its bits order like its value, NaN above all
             if (bin != INT_MAX) {
                 auto add = [&](const cufftDoubleComplex* r) {
                     if (!r) return;
                     const cufftDoubleComplex f = r[c];
                     const double u = f.x * f.x + f.y * f.y;
-                    p = SUM ? p + u : (u > p ? u : p);
+                    const unsigned long long ub = (unsigned long long)__double_as_longlong(u);
+                    if (SUM) p += u;
+                    else top = ub > top ? ub : top;
                 };
                 add(r0);
                 add(r1);
@@ -181,9 +184,7 @@ __global__ void __launch_bounds__(SPEC_THREADS)
             const int prev = __shfl_up_sync(0xffffffffu, bin, 1);
             const bool head = bin != INT_MAX && bin > 0 && (lane == 0 || prev != bin);
             if (!SUM) {
-                // p >= 0: its bit pattern orders like its value
-                const unsigned long long v = run_reduce<unsigned long long, true>(
-                    (unsigned long long)__double_as_longlong(p), same);
+                const unsigned long long v = run_reduce<unsigned long long, true>(top, same);
                 if (head) atomicMax(&spec_bins[bin - 1], v);
             } else {
                 // modes stored for both members of a pair count once
