@@ -17,6 +17,7 @@
 // (+-n_a, +-n_b, n_c)) and of |n| (unit 2^-28), so the result does not depend on the order
 // of the atomic additions.
 #include <dlfcn.h>
+#include <float.h>
 #include <limits.h>
 #include <math.h>
 #include <stdlib.h>
@@ -175,6 +176,20 @@ __global__ void __launch_bounds__(SPEC_THREADS)
                 add(r2);
                 add(r3);
             }
+            double unit = FIX_P;  // of p / maximum
+            if (SUM && p > DBL_MAX) {  // four finite squares, too large together: quarters
+                auto quarter = [&](const cufftDoubleComplex* r) {
+                    if (!r) return;
+                    const cufftDoubleComplex f = r[c];
+                    p += 0.25 * (f.x * f.x + f.y * f.y);
+                };
+                p = 0.0;
+                unit = 4.0 * FIX_P;
+                quarter(r0);
+                quarter(r1);
+                quarter(r2);
+                quarter(r3);
+            }
             bool same[5];
 #pragma unroll
             for (int e = 0; e < 5; e++) {
@@ -192,7 +207,7 @@ __global__ void __launch_bounds__(SPEC_THREADS)
                 unsigned long long ps = 0, ks = 0;
                 if (bin != INT_MAX && bin > 0) {
                     const double pm = __longlong_as_double((long long)maxbits[bin - 1]);
-                    ps = pm > 0.0 ? (unsigned long long)llrint(p / pm * FIX_P) * w : 0ull;
+                    ps = pm > 0.0 ? (unsigned long long)llrint(p / pm * unit) * w : 0ull;
                     const float rest = fmaf(-root, root, (float)d2) / (2.f * root);
                     ks = (unsigned long long)((long long)(root * (float)FIX_K) +
                                               llrintf(rest * (float)FIX_K)) *

@@ -41,3 +41,14 @@ def test_overflowing_transform_is_not_finite():
     P, _, n = B.sdot_power_spectrum(rho, 1.0, 12)
     assert np.all(n > 0)
     assert not np.isfinite(P[7:]).any(), P
+
+
+def test_point_mass_near_the_largest_double():
+    # |F_k|^2 = 1e308 for every mode: finite, but not the sum of the four modes (+-a, +-b, c).
+    # P is L^3 in every bin (tolerance: the transform's rounding and the fixed point's)
+    M, L = 16, 2.0
+    rho = np.zeros((M, M, M))
+    rho[3, 5, 7] = 1e154
+    P, _, n = B.sdot_power_spectrum(rho, L, M)
+    assert np.all(n[:13] > 0)
+    np.testing.assert_allclose(P[:13], L ** 3, rtol=1e-9, atol=0)
