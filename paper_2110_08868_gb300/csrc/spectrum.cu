@@ -121,8 +121,10 @@ __device__ __forceinline__ T run_reduce(T v, const bool (&same)[5]) {
 // third: up to four modes with one |n|, so one bin and one count. Along a row |n| does not
 // decrease over the lanes, so equal bins are runs, which are summed by shuffles before one
 // lane adds to the block's bins in shared memory; the block adds those to the global bins
-// once. The bin and |n| come from the integer |n|^2 in FP32 (a root and its residual: 48
-// bits), since FP64 is issued at a sixteenth of that rate.
+// once. The bin and |n| come from the integer |n|^2 without FP64, which is issued at a
+// sixteenth of FP32's rate: an FP32 root and its residual give |n| in 2^-28 to one unit, and
+// the integer |n|^2 2^56 - K^2 says which way the nearest unit K lies (an FP64 root rounds 6 of
+// the 786,432 integers up to the |n|^2 of M = 1024 the wrong way, the root and residual alone 116).
 // SUM = false: the largest |F_k|^2 per bin (bits in b0). SUM = true: b0 the sum of |F_k|^2
 // in units of the bin's maximum / 2^38, b1 that of |n| in 2^-28, b2 the mode count.
 // M = 512 (67 M modes, 1.08 GB read twice): maximum 4.6 -> 0.25 ms, sums 4.8 -> 0.51 ms, where
@@ -209,9 +211,14 @@ __global__ void __launch_bounds__(SPEC_THREADS)
                     const double pm = __longlong_as_double((long long)maxbits[bin - 1]);
                     ps = pm > 0.0 ? (unsigned long long)llrint(p / pm * unit) * w : 0ull;
                     const float rest = fmaf(-root, root, (float)d2) / (2.f * root);
-                    ks = (unsigned long long)((long long)(root * (float)FIX_K) +
-                                              llrintf(rest * (float)FIX_K)) *
-                         (w * rows);
+                    unsigned long long K = (unsigned long long)((long long)(root * (float)FIX_K) +
+                                                                llrintf(rest * (float)FIX_K));
+                    // (K - 1/2)^2 < |n|^2 2^56 < (K + 1/2)^2; |rest56| < 2^40, so 64 bits do
+                    const long long rest56 =
+                        (long long)(((unsigned long long)d2 << 56) - K * K);
+                    K += rest56 > (long long)K ? 1 : 0;
+                    K -= rest56 <= -(long long)K ? 1 : 0;
+                    ks = K * (w * rows);
                 }
                 ps = run_reduce<unsigned long long, false>(ps, same);
                 ks = run_reduce<unsigned long long, false>(ks, same);

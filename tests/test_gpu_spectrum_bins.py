@@ -1,7 +1,10 @@
-"""The binning of sdot_power_spectrum: meshes on both sides of the 33 values of the last
+"""The binning of sdot_power_spectrum: meshes on both sides of the 32 values of the last
 index that a warp's first round covers, the mean |k| to the last fixed-point unit, and
-transforms that overflow.
+transforms at the upper end of FP64 and beyond it.
 """
+import math
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -29,6 +32,35 @@ def test_binning_rounds_match_the_oracle(M):
         np.testing.assert_array_equal(n, no)
         np.testing.assert_allclose(P, Po, rtol=1e-9, atol=0)
         np.testing.assert_allclose(k, ko, rtol=1e-9, atol=0)
+
+
+def _k_units(M, nbins):
+    """Per bin the sum over its modes of |n| in units of 2^-28, each rounded to the nearest
+    (integer arithmetic throughout), and the mode counts."""
+    f = np.fft.fftfreq(M, d=1.0 / M).astype(np.int64) ** 2
+    d2 = np.bincount((f[:, None, None] + f[None, :, None] + f[None, None, :]).reshape(-1))
+    units, cnt = [0] * nbins, [0] * nbins
+    for v in np.flatnonzero(d2):
+        v, m = int(v), int(d2[v])
+        b = (math.isqrt(4 * v) + 1) // 2  # floor(sqrt(v) + 1/2)
+        if 1 <= b <= nbins:
+            r = (math.isqrt(v << 58) + 1) // 2  # sqrt(v) 2^28, rounded
+            units[b - 1] += m * r
+            cnt[b - 1] += m
+    return units, cnt
+
+
+@pytest.mark.parametrize("M", [31, 64, 200])
+def test_mean_k_to_the_last_unit(M):
+    # L = 2 pi: k is |n|. A bin's sum is below 2^52 units, so the one rounding of the mean
+    # (the division by the count) moves it by less than half a unit of the sum
+    nbins = 2 * M
+    _, k, n = B.sdot_power_spectrum(np.ones((M, M, M)), 2.0 * math.pi, nbins)
+    units, cnt = _k_units(M, nbins)
+    np.testing.assert_array_equal(n, cnt)
+    assert max(units) < 2 ** 52
+    got = [round(Fraction(float(kb)) * c * 2 ** 28) for kb, c in zip(k, cnt)]
+    assert got == units
 
 
 def test_overflowing_transform_is_not_finite():
