@@ -408,7 +408,7 @@ __device__ __noinline__ int poly_gc(int slot, int lane) {
     return nn;
 }
 
-enum { CLIP_NONE = 0, CLIP_CUT = 1, CLIP_EMPTY = 2, CLIP_CAP = 3, CLIP_BAD = 4 };
+enum { CLIP_NONE = 0, CLIP_CUT = 1, CLIP_EMPTY = 2, CLIP_CAP = 3, CLIP_BAD = 4, CLIP_TWICE = 8 };
 
 // relative tolerance of the vertex classification: a vertex counts as outside only
 // when it is beyond the plane by more than this fraction of the terms involved, so
@@ -448,8 +448,12 @@ __device__ __noinline__ bool poly_cut_by(int slot, V4<R> pn, R plen, int lane) {
 //    over a triangle's three edges ran the vertex arithmetic three times over).
 // First diagram of a 97^3 box, mixed: 219 -> 182 ms; FP64 evaluations of a 45^3 box, whose
 // vertex arithmetic fills the FP64 pipe: 31.6 -> 24.1 ms; the mesh deposit 92.7 -> 54.2 ms.
-template <typename R, class C>
-__device__ __noinline__ int poly_clip(int slot, V4<R> pn, R plen, int32_t j, int lane) {
+//
+// ONCE: a clip whose boundary would meet a face twice is refused (CLIP_TWICE, the polytope as
+// it was): the vertices of a face within rounding of the plane can lie on its two sides by
+// turns, and a list of plane triples cannot say which of the face's two new edges is which.
+template <typename R, class C, bool ONCE>
+__device__ __forceinline__ int clip_by(int slot, V4<R> pn, R plen, int32_t j, int lane) {
     Poly<R, C>& P = poly_at<R, C>(slot);
     constexpr int SL = C::SL, NW = C::NW;
     static_assert(sizeof(P.adj) <= 3 * C::MNEW * sizeof(R), "the table shares the new vertices");
@@ -527,6 +531,26 @@ __device__ __noinline__ int poly_clip(int slot, V4<R> pn, R plen, int32_t j, int
     }
     const int nkept = nt - nrem;
     if (nkept + nnew > C::MT || nnew > C::MNEW) return CLIP_CAP;
+    if (ONCE) {  // every boundary edge leaves another face
+        uint32_t from[NW];
+#pragma unroll
+        for (int q = 0; q < NW; q++) from[q] = 0u;
+        uint32_t bits = bmask;
+        for (int r = lane; r < nrem; r += 32, bits >>= 3) {
+            const uint32_t t = P.rem[r];
+#pragma unroll
+            for (int e = 0; e < 3; e++) {
+                const uint32_t x = (t >> (8 * e)) & 0xff;
+#pragma unroll
+                for (int q = 0; q < NW; q++)
+                    if (((bits >> e) & 1u) && (x >> 5) == q) from[q] |= 1u << (x & 31);
+            }
+        }
+        int faces = 0;
+#pragma unroll
+        for (int q = 0; q < NW; q++) faces += __popc(__reduce_or_sync(FULLMASK, from[q]));
+        if (faces != nnew) return CLIP_TWICE;
+    }
     // the boundary edges x -> y (in the order of the removed list), with the slot of the
     // removed vertex they leave
     for (int r = lane; r < nrem; r += 32, bmask >>= 3) {
@@ -621,6 +645,14 @@ __device__ __noinline__ int poly_clip(int slot, V4<R> pn, R plen, int32_t j, int
     lbad = __any_sync(FULLMASK, lbad);
     __syncwarp();
     return lbad ? CLIP_CUT | CLIP_BAD : CLIP_CUT;
+}
+template <typename R, class C>
+__device__ __noinline__ int poly_clip(int slot, V4<R> pn, R plen, int32_t j, int lane) {
+    return clip_by<R, C, false>(slot, pn, plen, j, lane);
+}
+template <typename R, class C>
+__device__ __noinline__ int poly_clip_once(int slot, V4<R> pn, R plen, int32_t j, int lane) {
+    return clip_by<R, C, true>(slot, pn, plen, j, lane);
 }
 
 // is seed j already one of the polytope's planes? (warp-uniform j)

@@ -83,8 +83,9 @@ __device__ __forceinline__ double wrap_rn(double dx, double L) {
 using MeshCap = Cap<64, 128, 8>;
 constexpr int MESH_MAXF = 26;
 
-// volume of polytope slot about its frame origin (units of a^3); 0 when a face is broken.
-// Every lane gets the value.
+// volume of polytope slot about its frame origin (units of a^3). Every lane gets the value.
+// NaN when the faces' cycles do not close: every entry of a face has to follow exactly one
+// other (rounding in near-degenerate clips can leave a vertex list that is no polytope).
 template <class C>
 __device__ __noinline__ double mesh_volume(int slot, int lane) {
     Poly<double, C>& P = poly_at<double, C>(slot);
@@ -131,30 +132,33 @@ __device__ __noinline__ double mesh_volume(int slot, int lane) {
     __syncwarp();
     double v6 = 0.0;
     bool ok = true;
-    for (int s = lane; s < nt; s += 32) {
-        const uint32_t t = P.tri[s];
-        const V3<double> v = vert(P, s);
+    unsigned taken = 0;  // sum of the entries that follow one
+    for (int s0 = 0; s0 < nt; s0 += 32) {
+        const int s = s0 + lane;
+        const bool act = s < nt;
+        const uint32_t t = act ? P.tri[s] : 0u;
+        const V3<double> v = vert(P, act ? s : 0);
 #pragma unroll 1
         for (int e = 0; e < 3; e++) {
             const uint32_t f = (t >> (8 * e)) & 0xff, y = (t >> (8 * ((e + 2) % 3))) & 0xff;
             // the next vertex of face f after s: its entry's first plane is y
-            int nx = -1;
-            for (int q = f > 0 ? (int)P.fend[f - 1] : 0; q < (int)P.fend[f]; q++)
-                if ((P.fent[q] & 0xff) == y) {
-                    nx = (int)(P.fent[q] >> 16);
-                    break;
-                }
-            if (nx < 0) {
-                ok = false;
-                continue;
-            }
-            const V3<double> w = vert(P, nx), r = vert(P, (int)ref[f]);
-            v6 += r.x * (v.y * w.z - v.z * w.y) + r.y * (v.z * w.x - v.x * w.z) +
-                  r.z * (v.x * w.y - v.y * w.x);
+            int q = f > 0 ? (int)P.fend[f - 1] : 0;
+            const int end = act ? (int)P.fend[f] : 0;
+            while (q < end && (P.fent[q] & 0xff) != y) q++;
+            __syncwarp();  // the lanes part in the search; the FP64 work is for all of them
+            const bool some = q < end;
+            ok = ok && (some || !act);
+            taken += some ? q : 0;
+            const V3<double> w = vert(P, some ? (int)(P.fent[q] >> 16) : 0), r = vert(P, (int)ref[f]);
+            const double d = r.x * (v.y * w.z - v.z * w.y) + r.y * (v.z * w.x - v.x * w.z) +
+                             r.z * (v.x * w.y - v.y * w.x);
+            if (some) v6 += d;
         }
     }
     v6 = warp_sum(v6);
-    return __all_sync(FULLMASK, ok) ? v6 * (1.0 / 6.0) : 0.0;
+    const unsigned n3 = 3u * (unsigned)nt;
+    ok = __reduce_add_sync(FULLMASK, taken) == n3 * (n3 - 1) / 2 && ok;
+    return __all_sync(FULLMASK, ok) ? v6 * (1.0 / 6.0) : NAN;
 }
 
 // bounds of the vertices along an axis, in FP32, a little outside
@@ -176,7 +180,10 @@ __device__ __forceinline__ void mesh_extent(int slot, int a, int lane, float& lo
 }
 
 // clip polytope slot by x_a <= b (up) or x_a >= b; false when nothing is left or, with bad
-// set, when the clip failed
+// set, when the clip failed. A plane within rounding of a facet, edge or cluster of vertices
+// can be refused (CLIP_TWICE): it is then moved aside by SHIFT, twice that, and so on (units
+// of a; the tolerance of beyond is 1e-13 of the terms) until it clears them.
+constexpr double SHIFT = 4e-13;
 template <class C>
 __device__ __forceinline__ bool mesh_cut(int slot, int a, double b, bool up, int lane, bool& bad,
                                          bool* cut = nullptr) {
@@ -186,7 +193,12 @@ __device__ __forceinline__ bool mesh_cut(int slot, int a, double b, bool up, int
     pn.y = a == 1 ? sg : 0.0;
     pn.z = a == 2 ? sg : 0.0;
     pn.w = sg * b;
-    const int r = poly_clip<double, C>(slot, pn, 1.0, -2, lane);
+    int r = poly_clip_once<double, C>(slot, pn, 1.0, -2, lane);
+    for (int k = 0; r == CLIP_TWICE && k < 14; k++) {
+        pn.w = sg * (b + (k & 1 ? -SHIFT : SHIFT) * (double)(1 << (k >> 1)));
+        r = poly_clip_once<double, C>(slot, pn, 1.0, -2, lane);
+    }
+    if (r == CLIP_TWICE) r = CLIP_CAP;
     if (cut) *cut = r != CLIP_NONE;
     if ((r & CLIP_BAD) || r == CLIP_CAP) bad = true;
     return r != CLIP_EMPTY && r != CLIP_CAP;
@@ -378,6 +390,10 @@ __global__ void __launch_bounds__(32)
                         const bool some = mesh_cut<C>(ys, 0, (double)vx * kk[0] + k0[0], true,
                                                       lane, bad, &cut);
                         below = !some ? 0.0 : (cut ? mesh_volume<C>(ys, lane) : left);
+                    }
+                    if (isnan(left) || isnan(below)) {  // a piece whose faces do not close
+                        bad = true;
+                        break;
                     }
                     const double mass = (left - below) * unit;
                     if (lane == 0 && mass > 0.0)
