@@ -531,26 +531,6 @@ __device__ __forceinline__ int clip_by(int slot, V4<R> pn, R plen, int32_t j, in
     }
     const int nkept = nt - nrem;
     if (nkept + nnew > C::MT || nnew > C::MNEW) return CLIP_CAP;
-    if (ONCE) {  // every boundary edge leaves another face
-        uint32_t from[NW];
-#pragma unroll
-        for (int q = 0; q < NW; q++) from[q] = 0u;
-        uint32_t bits = bmask;
-        for (int r = lane; r < nrem; r += 32, bits >>= 3) {
-            const uint32_t t = P.rem[r];
-#pragma unroll
-            for (int e = 0; e < 3; e++) {
-                const uint32_t x = (t >> (8 * e)) & 0xff;
-#pragma unroll
-                for (int q = 0; q < NW; q++)
-                    if (((bits >> e) & 1u) && (x >> 5) == q) from[q] |= 1u << (x & 31);
-            }
-        }
-        int faces = 0;
-#pragma unroll
-        for (int q = 0; q < NW; q++) faces += __popc(__reduce_or_sync(FULLMASK, from[q]));
-        if (faces != nnew) return CLIP_TWICE;
-    }
     // the boundary edges x -> y (in the order of the removed list), with the slot of the
     // removed vertex they leave
     for (int r = lane; r < nrem; r += 32, bmask >>= 3) {
@@ -561,6 +541,20 @@ __device__ __forceinline__ int clip_by(int slot, V4<R> pn, R plen, int32_t j, in
         if (bmask & 4u) P.ftri[pos++] = c | (a << 8) | (ps << 16) | sr;
     }
     __syncwarp();
+    if (ONCE) {  // every boundary edge leaves another face
+        uint32_t from[NW];
+#pragma unroll
+        for (int q = 0; q < NW; q++) from[q] = 0u;
+        for (int n = lane; n < nnew; n += 32) {
+            const uint32_t x = P.ftri[n] & 0xff;
+#pragma unroll
+            for (int q = 0; q < NW; q++) from[q] |= (x >> 5) == q ? 1u << (x & 31) : 0u;
+        }
+        int faces = 0;
+#pragma unroll
+        for (int q = 0; q < NW; q++) faces += __popc(__reduce_or_sync(FULLMASK, from[q]));
+        if (faces != nnew) return CLIP_TWICE;
+    }
     // new vertices: the point of the edge's two planes and the new plane; when that
     // system is ill-conditioned (the new plane almost parallel to the edge) the vertex
     // is interpolated on the edge between its kept and removed end points (the kept one

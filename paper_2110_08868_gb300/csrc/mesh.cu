@@ -20,18 +20,21 @@
 // One warp per cell. The cell is rebuilt in FP64 (seed frame) from its stored topology, or
 // from the facets of the context's last evaluation, which are its complete neighbour set.
 //
-// What bounds it is the FP64 pipe (a warp instruction every 16 cycles of an SM), so:
+// What bounds it is the chain of one warp's instructions, 7 warps an SM (12 cycles an
+// instruction, 3 of them fetching it; the FP64 pipe, a warp instruction every 16 cycles of an
+// SM, is 51% busy), so:
 //  - a cell is cut into z slabs, those into y slabs, and a y slab by the x planes from the
 //    top down in place, each piece the difference of two volumes: about 13 clips and 11
 //    volumes for a cell that meets 2.2 voxels an axis, where every voxel's six planes cut a
 //    copy of the whole cell (64 clips);
-//  - a volume is the sum of v_s.(v_next x r_f) over the vertices and their three faces (r_f:
-//    a vertex of the face): 27 FP64 operations a lane, with no chain along the faces;
+//  - a volume is a sum over the vertices and their three faces, with no chain along a face,
+//    of three FP64 operations each (mesh_volume);
 //  - a mesh point is tested against the planes in FP32, in FP64 only where that is too
 //    close to say;
 //  - the owner needs no second pass unless some point was claimed twice.
-// 110,592 cells, 96^3 points and voxels: 49.4 -> 12.6 ms (11.9 with
-// topo_init's FP32 test).
+// 110,592 cells, 96^3 points and voxels: 49.4 ms with the six planes of every voxel, 11.6 now.
+// Error of the density against exact clipping, 12^3 cells: the unit of |box| / 2^62 in which
+// masses are added, 7e-16 rms on 16^3 voxels, as with the six planes.
 #include <math.h>
 
 #include <string>
@@ -44,7 +47,7 @@ struct MeshParams {
     int M;                           // mesh points (voxels) per axis
     int pass;                        // 0: deposit, phi minimum, owner; 1: owner only
     double s;                        // 1 - lambda
-    double h[3];                     // voxel size
+    double h[3], inv_h[3];           // voxel size, its inverse
     double inv_unit;                 // 1 / fixed-point unit of the voxel masses
     const double* nu;                // masses (sorted order)
     const double* centre;            // 3 M: voxel centres (m + 1/2) L / M per axis
@@ -83,27 +86,26 @@ __device__ __forceinline__ double wrap_rn(double dx, double L) {
 using MeshCap = Cap<64, 128, 8>;
 constexpr int MESH_MAXF = 26;
 
+// a plane's axis and side
+__device__ __forceinline__ int32_t mesh_tag(int a, bool up) { return a | (up ? 0 : 4); }
+
 // volume of polytope slot about its frame origin (units of a^3). Every lane gets the value.
+// Faces are scaled to n_a = +-1 along their axis a, which pj holds (mesh_tag): 6 V is the sum
+// over the faces of +-w times twice the face's area seen along a, a sum of cross products of
+// consecutive vertices in two coordinates (three FP64 operations a vertex and face).
 // NaN when the faces' cycles do not close: every entry of a face has to follow exactly one
 // other (rounding in near-degenerate clips can leave a vertex list that is no polytope).
 template <class C>
 __device__ __noinline__ double mesh_volume(int slot, int lane) {
     Poly<double, C>& P = poly_at<double, C>(slot);
     const int nt = P.nt, np = P.np;
-    uint32_t* ref = reinterpret_cast<uint32_t*>(P.fa);  // lowest vertex of each face
-    for (int f = lane; f < np; f += 32) {
-        P.fend[f] = 0u;
-        ref[f] = 0xffu;
-    }
+    for (int f = lane; f < np; f += 32) P.fend[f] = 0u;
     __syncwarp();
     for (int s = lane; s < nt; s += 32) {
         const uint32_t t = P.tri[s];
-#pragma unroll
-        for (int e = 0; e < 3; e++) {
-            const uint32_t f = (t >> (8 * e)) & 0xff;
-            atomicAdd(&P.fend[f], 1u);
-            atomicMin(&ref[f], (uint32_t)s);
-        }
+        atomicAdd(&P.fend[t & 0xff], 1u);
+        atomicAdd(&P.fend[(t >> 8) & 0xff], 1u);
+        atomicAdd(&P.fend[(t >> 16) & 0xff], 1u);
     }
     __syncwarp();
     {
@@ -137,7 +139,6 @@ __device__ __noinline__ double mesh_volume(int slot, int lane) {
         const int s = s0 + lane;
         const bool act = s < nt;
         const uint32_t t = act ? P.tri[s] : 0u;
-        const V3<double> v = vert(P, act ? s : 0);
 #pragma unroll 1
         for (int e = 0; e < 3; e++) {
             const uint32_t f = (t >> (8 * e)) & 0xff, y = (t >> (8 * ((e + 2) % 3))) & 0xff;
@@ -149,10 +150,12 @@ __device__ __noinline__ double mesh_volume(int slot, int lane) {
             const bool some = q < end;
             ok = ok && (some || !act);
             taken += some ? q : 0;
-            const V3<double> w = vert(P, some ? (int)(P.fent[q] >> 16) : 0), r = vert(P, (int)ref[f]);
-            const double d = r.x * (v.y * w.z - v.z * w.y) + r.y * (v.z * w.x - v.x * w.z) +
-                             r.z * (v.x * w.y - v.y * w.x);
-            if (some) v6 += d;
+            const int tag = P.pj[f], a = tag & 3;
+            const int v = act ? s : 0, w = some ? (int)(P.fent[q] >> 16) : 0;
+            const double* u1 = a == 0 ? P.vy : (a == 1 ? P.vz : P.vx);
+            const double* u2 = a == 0 ? P.vz : (a == 1 ? P.vx : P.vy);
+            const double d = u1[v] * u2[w] - u2[v] * u1[w], h = P.pl[f].w;
+            if (some) v6 = fma(tag & 4 ? -h : h, d, v6);
         }
     }
     v6 = warp_sum(v6);
@@ -193,10 +196,10 @@ __device__ __forceinline__ bool mesh_cut(int slot, int a, double b, bool up, int
     pn.y = a == 1 ? sg : 0.0;
     pn.z = a == 2 ? sg : 0.0;
     pn.w = sg * b;
-    int r = poly_clip_once<double, C>(slot, pn, 1.0, -2, lane);
+    int r = poly_clip_once<double, C>(slot, pn, 1.0, mesh_tag(a, up), lane);
     for (int k = 0; r == CLIP_TWICE && k < 14; k++) {
         pn.w = sg * (b + (k & 1 ? -SHIFT : SHIFT) * (double)(1 << (k >> 1)));
-        r = poly_clip_once<double, C>(slot, pn, 1.0, -2, lane);
+        r = poly_clip_once<double, C>(slot, pn, 1.0, mesh_tag(a, up), lane);
     }
     if (r == CLIP_TWICE) r = CLIP_CAP;
     if (cut) *cut = r != CLIP_NONE;
@@ -339,27 +342,38 @@ __global__ void __launch_bounds__(32)
             P.vy[s] -= c[1];
             P.vz[s] -= c[2];
         }
-        for (int k = lane; k < P.np; k += 32)
-            P.pl[k].w -= P.pl[k].x * c[0] + P.pl[k].y * c[1] + P.pl[k].z * c[2];
+        // and the planes are scaled to a largest component of 1 (mesh_volume)
+        for (int k = lane; k < P.np; k += 32) {
+            V4<double> n = P.pl[k];
+            const double nx = fabs(n.x), ny = fabs(n.y), nz = fabs(n.z);
+            const int a = nx >= ny && nx >= nz ? 0 : (ny >= nz ? 1 : 2);
+            const double sc = 1.0 / (a == 0 ? nx : (a == 1 ? ny : nz));
+            n.w = (n.w - (n.x * c[0] + n.y * c[1] + n.z * c[2])) * sc;
+            n.x = a == 0 ? copysign(1.0, n.x) : n.x * sc;
+            n.y = a == 1 ? copysign(1.0, n.y) : n.y * sc;
+            n.z = a == 2 ? copysign(1.0, n.z) : n.z * sc;
+            P.pl[k] = n;
+            P.plen[k] *= sc;
+            P.pj[k] = mesh_tag(a, (a == 0 ? n.x : (a == 1 ? n.y : n.z)) > 0.0);
+        }
         __syncwarp();
         const double volP = mesh_volume<C>(ps, lane);
         if (!(volP > 0.0)) {
             if (lane == 0) atomicAdd(mp.flags, 1);
             continue;
         }
-        // voxel edge v along axis a, pulled back to the cell's frame: v k[a] + k0[a]
+        // voxel edge v along axis a, pulled back to the cell's frame. The difference v h - y
+        // comes first: scaled apart, the two lose what they cancel (N^(1/3) units in the
+        // last place of a, and the masses on the plane's two sides with it)
         const double ks = 1.0 / (mp.s * cp.a);
-        double kk[3], k0[3];
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            kk[a] = mp.h[a] * ks;
-            k0[a] = -y[a] * ks - c[a];
-        }
+        auto edge = [&](int a, long long v) { return fma((double)v, mp.h[a], -y[a]) * ks - c[a]; };
         auto range = [&](int slot, int a, long long& va, long long& vb) {
             float l, h;
             mesh_extent<C>(slot, a, lane, l, h);
-            va = (long long)floor(((double)l - k0[a]) / kk[a]);
-            vb = (long long)floor(((double)h - k0[a]) / kk[a]);
+            const double sa = mp.s * cp.a;
+            // (l and h lie outside by far more than the rounding of the product)
+            va = (long long)floor(fma((double)l + c[a], sa, y[a]) * mp.inv_h[a]);
+            vb = (long long)floor(fma((double)h + c[a], sa, y[a]) * mp.inv_h[a]);
         };
         const double unit = mp.nu[i] / volP * mp.inv_unit;  // fixed-point mass per volume
         bool bad = false;
@@ -367,17 +381,17 @@ __global__ void __launch_bounds__(32)
         range(ps, 2, z0, z1);
         for (long long vz = z0; vz <= z1; vz++) {
             poly_copy<double, C>(zs, ps, lane);
-            if (vz > z0 && !mesh_cut<C>(zs, 2, (double)vz * kk[2] + k0[2], false, lane, bad)) continue;
-            if (vz < z1 && !mesh_cut<C>(zs, 2, (double)(vz + 1) * kk[2] + k0[2], true, lane, bad))
+            if (vz > z0 && !mesh_cut<C>(zs, 2, edge(2, vz), false, lane, bad)) continue;
+            if (vz < z1 && !mesh_cut<C>(zs, 2, edge(2, vz + 1), true, lane, bad))
                 continue;
             long long y0, y1;
             range(zs, 1, y0, y1);
             for (long long vy = y0; vy <= y1; vy++) {
                 poly_copy<double, C>(ys, zs, lane);
-                if (vy > y0 && !mesh_cut<C>(ys, 1, (double)vy * kk[1] + k0[1], false, lane, bad))
+                if (vy > y0 && !mesh_cut<C>(ys, 1, edge(1, vy), false, lane, bad))
                     continue;
                 if (vy < y1 &&
-                    !mesh_cut<C>(ys, 1, (double)(vy + 1) * kk[1] + k0[1], true, lane, bad))
+                    !mesh_cut<C>(ys, 1, edge(1, vy + 1), true, lane, bad))
                     continue;
                 long long x0, x1;
                 range(ys, 0, x0, x1);
@@ -387,7 +401,7 @@ __global__ void __launch_bounds__(32)
                     double below = 0.0;
                     if (vx > x0) {
                         bool cut;
-                        const bool some = mesh_cut<C>(ys, 0, (double)vx * kk[0] + k0[0], true,
+                        const bool some = mesh_cut<C>(ys, 0, edge(0, vx), true,
                                                       lane, bad, &cut);
                         below = !some ? 0.0 : (cut ? mesh_volume<C>(ys, lane) : left);
                     }
@@ -467,7 +481,10 @@ int mesh_eval(DeviceState& d, int M, double lambda, double* rho_dev, double* phi
     MeshParams mp;
     mp.M = M;
     mp.s = 1.0 - lambda;
-    for (int a = 0; a < 3; a++) mp.h[a] = d.L[a] / M;
+    for (int a = 0; a < 3; a++) {
+        mp.h[a] = d.L[a] / M;
+        mp.inv_h[a] = M / d.L[a];
+    }
     const double mass_unit = d.L[0] * d.L[1] * d.L[2] / 4611686018427387904.0;  // |box| / 2^62
     mp.inv_unit = 1.0 / mass_unit;
     mp.nu = d.nu;

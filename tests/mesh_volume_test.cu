@@ -29,7 +29,7 @@ __global__ void volumes(double* out) {
             P.pl[lane] = V4<double>{a == 0 ? s : 0.0, a == 1 ? s : 0.0, a == 2 ? s : 0.0,
                                     1.0 + s * o[a]};
             P.plen[lane] = 1.0;
-            P.pj[lane] = -1;
+            P.pj[lane] = mesh_tag(a, s > 0.0);
         }
         if (lane < 8) {  // corner (x, y, z), its planes ordered so that their normals turn right
             const int x = lane & 1, y = (lane >> 1) & 1, z = lane >> 2;
