@@ -30,8 +30,7 @@ namespace sdot {
 constexpr int CARRY_WARPS = 8;   // warps of a block
 constexpr int CARRY_BLOCKS = 4;  // blocks per SM the registers are sized for
 constexpr int MAXF = 26;         // facets (with the 6 box planes, one face a lane)
-constexpr int NPL = 32;          // planes a lane round builds: facets, then certificate seeds
-constexpr int NPL2 = MAXF + CERT_NEAR;
+constexpr int NPL2 = MAXF + CERT_NEAR;  // planes: facets, then certificate seeds
 
 struct CarryCell {
     V4<float> pl[NPL2];
@@ -290,14 +289,17 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
     for (int a = 0; a < 3; a++) o[a] = 0.5f * (redux_min(mn[a]) + redux_max(mx[a]));
     ill = __any_sync(FULLMASK, ill);
     __syncwarp();
-    // one face a lane: the fan of its lowest vertex, along the cycle of the dual edges
-    // (integrate's sums, in its order)
+    // one face a lane: the fan of its lowest vertex, along the cycle of the dual edges.
+    // Facet f is on lane 6 + f, where integrate has it (its slot, after the 6 box planes), so
+    // that the sums over the lanes below are integrate's in its order.
+    const int f = lane - 6;
+    const bool face = f >= 0 && f < nf;
     float fv6 = 0.f, fmx = 0.f, fmy = 0.f, fmz = 0.f, Sx = 0.f, Sy = 0.f, Sz = 0.f;
     int steps = 0;
     float coef = -1.f;
     float A = 0.f;
-    if (lane < nf) {
-        const uint32_t st = S.start[lane];
+    if (face) {
+        const uint32_t st = S.start[f];
         if (st == 0xffffffffu) {
             ok = false;
         } else {
@@ -309,7 +311,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
             v0.z = S.vz[s0] - o[2];
             V3<float> vp = v0;
             for (steps = 1; steps <= nt; steps++) {
-                const uint32_t e = S.edge[lane * MAXF + y];
+                const uint32_t e = S.edge[f * MAXF + y];
                 if (e == 0xffffu) {
                     ok = false;
                     break;
@@ -330,7 +332,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
             Sx = ax2;
             Sy = ay2;
             Sz = az2;
-            coef = A / S.plen[lane];
+            coef = A / S.plen[f];
             if (steps < 3 || !(A > 0.f)) ok = false;  // fewer facets than the topology has
         }
     }
@@ -366,7 +368,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
         if (dz2 > REFRAME_DIST * REFRAME_DIST) return false;
     }
     // outputs (the facet list, the topology and their counts stay as they are)
-    if (lane < nf) cp.fval[i * FCAP + lane] = (double)coef * cp.a;
+    if (face) cp.fval[i * FCAP + f] = (double)coef * cp.a;
     if ((lane & 7) == 0) {
         const double a3 = cp.a * cp.a * cp.a;
         if (quant == 0) {
