@@ -4,11 +4,13 @@
 // Near convergence 95 to 99% of the cells keep their topology and their certificate. For
 // them an evaluation is: planes at the new psi, vertices, the checks, the integrals. The
 // general pass (process_cell) does that too, and this kernel does the same arithmetic in
-// the same order, to the same bits; but a block there waits for its slowest cell, and a
-// cell whose topology broke is clipped from the box meanwhile. Here every cell does the
-// same short work, and whatever does not fit it (a broken topology, a certificate that
-// no longer holds, more than MAXF facets, a cell far from its frame) goes to a queue that
-// the general pass then takes, from scratch: nothing is written before a cell is through.
+// the same order (the geometry is the same inline code, the lengths and plane offsets name
+// their roundings; a test compares the two passes bit for bit); but a block there waits for
+// its slowest cell, and a cell whose topology broke is clipped from the box meanwhile. Here
+// every cell does the same short work, and whatever does not fit it (a broken topology, a
+// certificate that no longer holds, more than MAXF facets, a cell far from its frame) goes
+// to a queue that the general pass then takes, from scratch: nothing is written before a
+// cell is through.
 //
 // What bounds it: GB300 issues an FP64 warp instruction every 16 cycles of an SM, and the
 // general path used about 120 a cell (the plane offsets, warp sums of four FP64 totals, a
@@ -41,13 +43,7 @@ struct CarryCell {
     float sup[28];                    // stored supports less the margin
 };
 
-// sqrt(x x + y y + z z) with the rounding the general path's expression is compiled to, so
-// that a cell's facet coefficients are the same whichever pass takes it
-__device__ __forceinline__ float length_as_built(float x, float y, float z) {
-    return sqrtf(__fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y))));
-}
-
-// s + e = a + b exactly
+// s + e = a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ float two_sum(float a, float b, float& e) {
     const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
@@ -207,7 +203,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
         if (j >= 0 && j < cp.N && j != (int32_t)i) ok = plane_pair(cp, si, j, pn) && ok;
         else ok = false;
         S.pl[k] = pn;
-        S.plen[k] = length_as_built(pn.x, pn.y, pn.z);
+        S.plen[k] = length3(pn.x, pn.y, pn.z);
     }
     if (lane < 27)
         S.sup[lane] = lane == 13 ? INFINITY
@@ -328,7 +324,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
                 vp = vc;
             }
             const float ax2 = 0.5f * Sx, ay2 = 0.5f * Sy, az2 = 0.5f * Sz;
-            A = length_as_built(ax2, ay2, az2);
+            A = length3(ax2, ay2, az2);
             Sx = ax2;
             Sy = ay2;
             Sz = az2;
@@ -342,7 +338,7 @@ __device__ __forceinline__ bool carry_cell(CarryCell& S, const ClipParams& cp, i
     const float cs = warp_sum4(Sx, Sy, Sz, A, lane);
     const float sx = __shfl_sync(FULLMASK, cs, 0), sy = __shfl_sync(FULLMASK, cs, 8),
                 sz = __shfl_sync(FULLMASK, cs, 16), sabs = __shfl_sync(FULLMASK, cs, 24);
-    const bool bad = ill || !(sqrt(sx * sx + sy * sy + sz * sz) <= 1e-4f * sabs);
+    const bool bad = ill || !(length3(sx, sy, sz) <= 1e-4f * sabs);
     // totals, one quantity a lane: volume, then the moment about o carried to the seed
     const int quant = lane >> 3, ax = quant > 0 ? quant - 1 : 0;
     const double tot = warp_sum4((double)fv6, (double)fmx, (double)fmy, (double)fmz, lane);

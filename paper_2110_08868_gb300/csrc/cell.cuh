@@ -305,6 +305,16 @@ __device__ __noinline__ void poly_init(int slot, const ClipParams& cp, int lane)
     __syncwarp();
 }
 
+// |(x, y, z)|. In FP32 with its roundings named: facet coefficients are quotients of two of
+// these, and the carried pass (carry.cu) gives the same as the general one however the
+// compiler contracts either.
+__device__ __forceinline__ float length3(float x, float y, float z) {
+    return sqrtf(__fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y))));
+}
+__device__ __forceinline__ double length3(double x, double y, double z) {
+    return sqrt(x * x + y * y + z * z);
+}
+
 // The vertex of three planes; well: the triple is well conditioned,
 // det(n_a, n_b, n_c) > dtol |n_a| |n_b| |n_c|.
 template <typename R>
@@ -964,7 +974,7 @@ __device__ __forceinline__ void build_plane(const ClipParams& cp, const CellCtx&
         pn.z = (R)nz;
         pn.w = (R)w;
     }
-    plen = sqrt(pn.x * pn.x + pn.y * pn.y + pn.z * pn.z);
+    plen = length3(pn.x, pn.y, pn.z);
 }
 
 template <typename R>
@@ -1571,7 +1581,7 @@ __device__ __noinline__ uint32_t integrate(int slot, const ClipParams& cp, int l
         my += (double)fmy;
         mz += (double)fmz;
         const R ax2 = R(0.5) * Sx, ay2 = R(0.5) * Sy, az2 = R(0.5) * Sz;
-        const R A = sqrt(ax2 * ax2 + ay2 * ay2 + az2 * az2);
+        const R A = length3(ax2, ay2, az2);
         sx += ax2;
         sy += ay2;
         sz += az2;
@@ -1628,7 +1638,7 @@ __device__ __noinline__ uint32_t integrate(int slot, const ClipParams& cp, int l
         else cp.topo[i * TOPO + s2] = pack3(a, b2, c);
     }
     tok = __all_sync(FULLMASK, tok);
-    const R closure = sqrt(sx * sx + sy * sy + sz * sz);
+    const R closure = length3(sx, sy, sz);
     const R tol = sizeof(R) == 4 ? R(1e-4) : R(1e-10);
     if (!(closure <= tol * sabs)) bad = true;
     const double vol = vol6 * (1.0 / 6.0);
