@@ -290,7 +290,7 @@ int sdot_power_spectrum(const double* rho, int M, double L, int nbins, double* P
  *          order; the lowest index when the centre lies on a facet).
  * The device buffers it needs (16 M^3 bytes, plus staging for host outputs) come from
  * the context's allocator and are kept for the next call. SDOT_ERR_CAPACITY if a cell
- * cannot be rebuilt from its facets in the large polytope.
+ * cannot be rebuilt from its facets in the large polytope, or not be cut along the voxels.
  */
 int sdot_mesh(sdot_ctx* ctx, double lambda, int mesh, double* rho, double* phi,
               int32_t* owner);

@@ -1,5 +1,5 @@
 // One Laguerre cell per warp: the polytope, its clipping, the security walk and the
-// integrals. Included by clip.cu only.
+// integrals. Included by clip.cu, carry.cu and mesh.cu.
 //
 // Cell i of eq. (laguerrecell) in seed-local coordinates p = q - y_i is
 //     P_i = { p : p.d_ij <= b_ij for all j },  d_ij = minimum image of y_j - y_i,

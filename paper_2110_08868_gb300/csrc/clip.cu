@@ -22,8 +22,9 @@ int launch_carry(const ClipParams& cp, int32_t* queue, int32_t* cnt, int32_t* wo
 // A block's warps go through the phases of a cell together (see process_cell). Larger
 // blocks keep the instruction cache better, smaller ones wait less for their slowest cell.
 // 1, 2, 4, 8 blocks per SM (32 to 4 warps each): first diagram 97^3, whose cells differ
-// most, 191, 148, 132, 138 ms; early Newton step 100^3 119, 111, 121, 146 ms; late step
-// 129^3 75, 60, 53, 55 ms.
+// most, 177, 132, 113, 119 ms; early Newton step 100^3 95, 90, 105, 131 ms; late step 129^3
+// (1% of its cells left to these kernels) 17.4, 17.2, 17.3, 17.4 ms; FP64 step 45^3 15.2, 14.0,
+// 14.3, 16.4 ms.
 constexpr int CLIP_BLOCKS_PER_SM = 4;
 
 // Warps of a full clipping block: as many as shared memory holds polytopes for with

@@ -75,7 +75,8 @@ struct DeviceState {
     double a;                 // length unit: (|box| / N)^(1/3)
     // seeds
     Pos4* pos;             // sorted positions; w = caller index (exact in fp64)
-    float4* posf;             // (offset in grid cell / a, psi/a^2 hi), per evaluation
+    float4* posf;             // offset in grid cell / a (once a context), psi/a^2 hi (each
+                              // evaluation); before the first one scratch of the kNN build
     float* pslo;              // psi/a^2 lo part (psi/a^2 = hi + lo)
     uint4* ioff;              // offset in the grid cell as 32-bit fixed point (x, y, z, 0)
     int32_t* leafc;           // grid cell of each seed: x | y << 10 | z << 20
@@ -201,8 +202,11 @@ int build_pyramid(DeviceState& d, const double* psi, cudaStream_t s);
 int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult* res,
                    cudaStream_t s);
 // Batched evaluation of n contexts (one persistent launch per pass for all of their
-// cells; results identical to evaluate_cells on each context). The scratch holds the
-// job tables for up to cap contexts.
+// cells): each context's cells as evaluate_cells has them, except that the FP64 re-clip takes
+// the large polytope for every cell, where evaluate_cells takes the small one first. A cell
+// of that pass then walks although its certificate holds, and one that drops planes on the
+// way (over 58 live ones) can differ in the last places of its FP64 sums. The scratch holds
+// the job tables for up to cap contexts.
 struct BatchScratch;
 int batch_scratch_create(int cap, BatchScratch** out);
 void batch_scratch_destroy(BatchScratch* b);

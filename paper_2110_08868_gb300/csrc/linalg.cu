@@ -499,10 +499,10 @@ __global__ void cg_init_kernel(const double* __restrict__ nu, const double* __re
 //
 // W entries of a row are in flight at a time. A full wave of blocks hides the gathers'
 // latency behind its other warps with W = 8. A grid that is resident at once with two
-// blocks per SM (below 78 k rows) is one chain of latencies: W = 24 asks for nearly every row's entries at once, the scalars
-// of the last iteration are loaded at the start, and the launch overlaps the kernel before
-// (programmatic dependent launch). 4096 rows:
-// 23 -> 13.5 us an iteration, SpMV 21.7 -> 11.6.
+// blocks per SM (below 78 k rows) is one chain of latencies: W = 24 asks for nearly every
+// row's entries at once, the scalars of the last iteration are loaded at the start, and the
+// launch overlaps the kernel before (programmatic dependent launch). 4096 rows: SpMV
+// 21.7 -> 11.6 us (iterations: see cg_solve).
 template <int W>
 __global__ void __launch_bounds__(CG_THREADS, W == 8 ? 8 : 2)
     cg_spmv_kernel(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col,
@@ -730,14 +730,16 @@ int cg_solve(DeviceState& d, double rtol, int maxit, int* iters, double* rel_res
     NvtxRange nv("cg");
     const int64_t N = d.N;
     const int64_t nslice = (N + 31) / 32;
-    // memory-bound loops, one resident wave of 256-thread blocks; below a wave (311 k rows)
-    // only the blocks that have rows: 8 slices or 256 rows each in both kernels, so the
-    // partials and their order are those of the full grid (4096 rows: update 7.6 -> 5.6
-    // us, SpMV 23.4 -> 21.7)
+    // memory-bound loops, one resident wave of 256-thread blocks (5 an SM by the update's 48
+    // registers: 760 blocks); below a wave (194,560 rows) only the blocks that have rows: 8
+    // slices or 256 rows each in both kernels, so the partials and their order are those of
+    // the full grid (4096 rows: update 7.6 -> 5.6 us, SpMV 23.4 -> 21.7)
     const int64_t rows_nb = (N + CG_THREADS - 1) / CG_THREADS;
     const int wave = cg_blocks_per_sm() * num_sms();
     const int nb = (int)(rows_nb < wave ? rows_nb : wave);
-    // 64^3 rows (1024 blocks): 34.7 us an iteration with W = 8, 36.1 with 24
+    // an iteration with W = 8 / with W = 24 and overlapping launches: 16 blocks 22.1 / 15.8 us,
+    // 128: 22.5 / 19.7, 250: 25.0 / 22.0, 333: 25.6 / 22.3, 432: 25.4 / 26.3, 550: 27.6 / 26.9,
+    // 760 (64^3 rows) 35.4 / 35.0: a gain up to two blocks an SM, no clear one above
     const bool small = nb <= 2 * num_sms();
     cudaLaunchAttribute overlap;
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
