@@ -16,8 +16,8 @@ reserves; ``extra.eval_detail.carried`` counts the carried cells, and
 ``extra.cells_per_s_walk_only`` times the same calls on a context with carrying off.
 ``roofline`` is the first clipping pass against the derived FP32 peak, and
 ``extra.roofline_cg`` is the CG iteration against the measured HBM bandwidth. Their
-``traffic`` fields are DRAM bytes from ncu captures of the current kernels on the 128^3
-version of the box, scaled to a launch.
+``traffic`` fields are DRAM bytes from ncu captures of the current kernels on a 128^3 box,
+scaled to a launch (null: none since the kernel last changed).
 The default workload is the 256^3 Zel'dovich box with 5% clumped points (17.6 M
 seeds), mixed precision. ``--impl reference`` times the CPU oracle instead on a
 bounded sample of the same workload (certified cells at psi = 0, cells/s).
@@ -56,12 +56,12 @@ N_SM = 152
 CG_BYTES_PER_ROW = 124
 # per off-diagonal entry of L: int32 column + FP32 weight
 CG_BYTES_PER_ENTRY = 8
-# DRAM bytes (read + write) per unit from ncu captures of the current kernels on the
-# clumpy 128^3 box (N = 2,202,087), scaled to a launch by the units it processes (None:
-# not captured since the kernel last changed): the first clipping pass per cell, one CG
-# iteration (SpMV 402.4 MB + update 162.8 MB) per row
+# DRAM bytes (read + write) per unit from ncu captures of the current kernels, scaled to a
+# launch by the units it processes (None: not captured since the kernel last changed): the
+# first clipping pass per cell; one CG iteration per row, on a 128^3 box without clumps
+# (N = 2,097,152: SpMV 379.8 MB, update 155.7 MB)
 CLIP_DRAM_PER_CELL = None
-CG_DRAM_PER_ROW = (385.858560e6 + 16.551168e6 + 123.337216e6 + 39.467264e6) / 2202087
+CG_DRAM_PER_ROW = (364.542976e6 + 15.292928e6 + 117.574144e6 + 38.082816e6) / 2097152
 
 
 def parse():

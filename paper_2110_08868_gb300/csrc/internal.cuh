@@ -204,9 +204,9 @@ int evaluate_cells(DeviceState& d, const double* psi, int precision, EvalResult*
 // Batched evaluation of n contexts (one persistent launch per pass for all of their
 // cells): each context's cells as evaluate_cells has them, except that the FP64 re-clip takes
 // the large polytope for every cell, where evaluate_cells takes the small one first. A cell
-// of that pass then walks although its certificate holds, and one that drops planes on the
-// way (over 58 live ones) can differ in the last places of its FP64 sums. The scratch holds
-// the job tables for up to cap contexts.
+// of that pass then walks although its certificate holds, and one that uses up the small
+// polytope's plane slots on the way can differ in the last places of its FP64 sums. The
+// scratch holds the job tables for up to cap contexts.
 struct BatchScratch;
 int batch_scratch_create(int cap, BatchScratch** out);
 void batch_scratch_destroy(BatchScratch* b);
