@@ -22,7 +22,7 @@
 //
 // What bounds it is the chain of one warp's instructions, 7 warps an SM (12 cycles an
 // instruction, 3 of them fetching it; the FP64 pipe, a warp instruction every 16 cycles of an
-// SM, is 51% busy), so:
+// SM, is 53% busy), so:
 //  - a cell is cut into z slabs, those into y slabs, and a y slab by the x planes from the
 //    top down in place, each piece the difference of two volumes: about 13 clips and 11
 //    volumes for a cell that meets 2.2 voxels an axis, where every voxel's six planes cut a
